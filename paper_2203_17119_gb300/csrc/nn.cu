@@ -13,6 +13,7 @@
 // even sites and the output is read on odd sites.  Backward: g_psi_d =
 // T_d^+ g_z, gW2[d][b] = sum g_psi_d phi_b^+, g_phi_b = sum_d W2[d][b]^+ g_psi_d,
 // gW1[a][d] = sum g_phi_a R_d^+ (sums over sites, colour and lanes).
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -27,16 +28,15 @@ constexpr int kNDir = 11;
 constexpr int kAdj[kNDir] = {0, 5, 6, 7, 8, 1, 2, 3, 4, 10, 9};
 
 struct TransArgs {
-    const float* in;           // full field (both parities)
-    float* out;                // out fields, stride `fstride` floats
-    const float* const* ins;   // transport-sum: input field per direction
+    const float* same;         // parity-p block of the input (field 0)
+    const float* opp;          // parity-(1-p) block of the input (field 0)
+    float* out;                // parity-p block of the output (field 0)
     const float* links;        // FP32 doubled link table of parity p
     const int* nbr;
     const int4* tiles;
-    int dirs[kNDir];           // direction applied for output j
-    int ndir, N5, Ls, parity;
-    int64_t off_p, off_q;      // float offsets of parity p / 1-p blocks in a full field
-    int64_t fstride;           // floats per full field
+    int dirs[kNDir];           // direction of output (multi) or input (sum) field j
+    int ndir, N5, Ls;
+    int64_t istride, ostride;  // floats between consecutive input (sum) / output (multi) fields
 };
 
 // f = U v (3x3 complex times colour vector) for 4 spins
@@ -60,9 +60,11 @@ __device__ __forceinline__ void su3_spinor(const float* __restrict__ w, const fl
         }
 }
 
-// Value of T_d f at (site, lane) of parity p: 12 complex.
-__device__ __forceinline__ void transport_at(const TransArgs& a, const float* __restrict__ f, int d,
-                                             int64_t site, int tsite_nb_k, int lane,
+// Value of T_d f at (site, lane) of parity p: 12 complex; same / opp are f's
+// blocks of parity p and 1 - p (the link directions read only the latter, the
+// others only the former).
+__device__ __forceinline__ void transport_at(const TransArgs& a, const float* __restrict__ same,
+                                             const float* __restrict__ opp, int d, int64_t site, int lane,
                                              float (&orr)[12], float (&oi)[12]) {
     const int N5 = a.N5;
     if (d == 0 || d == 9 || d == 10) {
@@ -76,7 +78,7 @@ __device__ __forceinline__ void transport_at(const TransArgs& a, const float* __
             }
             l = d == 9 ? lane + 1 : lane - 1;
         }
-        const float* p = f + a.off_p + (site * 12 * N5 + l) * 2;
+        const float* p = same + (site * 12 * N5 + l) * 2;
 #pragma unroll
         for (int c = 0; c < 12; ++c) {
             const float2 v = *reinterpret_cast<const float2*>(p + (int64_t)c * N5 * 2);
@@ -92,9 +94,8 @@ __device__ __forceinline__ void transport_at(const TransArgs& a, const float* __
         for (int c = 0; c < 12; ++c) orr[c] = oi[c] = 0.f;
         return;
     }
-    (void)tsite_nb_k;
     float vr[12], vi[12];
-    const float* p = f + a.off_q + ((int64_t)n * 12 * N5 + lane) * 2;
+    const float* p = opp + ((int64_t)n * 12 * N5 + lane) * 2;
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
         const float2 v = *reinterpret_cast<const float2*>(p + (int64_t)c * N5 * 2);
@@ -104,7 +105,7 @@ __device__ __forceinline__ void transport_at(const TransArgs& a, const float* __
     su3_spinor(a.links + (site * 8 + k) * 18, vr, vi, orr, oi);
 }
 
-// out[j] = T_{dirs[j]} in on the sites of parity p (one thread per site x lane)
+// out field j = T_{dirs[j]} in on the sites of parity p (one thread per site x lane)
 __global__ void __launch_bounds__(256) k_transport_multi(const TransArgs a) {
     const int4 tl = a.tiles[blockIdx.x];
     const int N5 = a.N5;
@@ -113,8 +114,8 @@ __global__ void __launch_bounds__(256) k_transport_multi(const TransArgs a) {
         const int lane = t % N5;
         for (int j = 0; j < a.ndir; ++j) {
             float orr[12], oi[12];
-            transport_at(a, a.in, a.dirs[j], site, 0, lane, orr, oi);
-            float* o = a.out + j * a.fstride + a.off_p + (site * 12 * N5 + lane) * 2;
+            transport_at(a, a.same, a.opp, a.dirs[j], site, lane, orr, oi);
+            float* o = a.out + j * a.ostride + (site * 12 * N5 + lane) * 2;
 #pragma unroll
             for (int c = 0; c < 12; ++c)
                 *reinterpret_cast<float2*>(o + (int64_t)c * N5 * 2) = make_float2(orr[c], oi[c]);
@@ -122,7 +123,9 @@ __global__ void __launch_bounds__(256) k_transport_multi(const TransArgs a) {
     }
 }
 
-// out = sum_j T_{dirs[j]} ins[j] on the sites of parity p
+// out = sum_j T_{dirs[j]} in_j on the odd sites; in_j is input field j of the
+// block that direction reads (odd for 0, 9, 10, even for the links), counted
+// from 0 within each block
 __global__ void __launch_bounds__(256) k_transport_sum(const TransArgs a) {
     const int4 tl = a.tiles[blockIdx.x];
     const int N5 = a.N5;
@@ -132,13 +135,17 @@ __global__ void __launch_bounds__(256) k_transport_sum(const TransArgs a) {
         float ar[12], ai[12];
 #pragma unroll
         for (int c = 0; c < 12; ++c) ar[c] = ai[c] = 0.f;
+        int js = 0, jo = 0;
         for (int j = 0; j < a.ndir; ++j) {
             float orr[12], oi[12];
-            transport_at(a, a.ins[j], a.dirs[j], site, 0, lane, orr, oi);
+            const int d = a.dirs[j];
+            const bool link = d >= 1 && d <= 8;
+            const int64_t f = (link ? jo++ : js++) * a.istride;
+            transport_at(a, a.same + f, a.opp + f, d, site, lane, orr, oi);
 #pragma unroll
             for (int c = 0; c < 12; ++c) { ar[c] += orr[c]; ai[c] += oi[c]; }
         }
-        float* o = a.out + a.off_p + (site * 12 * N5 + lane) * 2;
+        float* o = a.out + (site * 12 * N5 + lane) * 2;
 #pragma unroll
         for (int c = 0; c < 12; ++c)
             *reinterpret_cast<float2*>(o + (int64_t)c * N5 * 2) = make_float2(ar[c], ai[c]);
@@ -199,83 +206,147 @@ __global__ void __launch_bounds__(128) k_mix(const float* __restrict__ in, int n
     }
 }
 
-// Weight gradient: g[o][so][i][si] = sum_pixels gout[o][so] conj(in[i][si]).
-// One thread per (o, i) pair with a 4x4 complex accumulator; the CTA walks
-// (site, colour) chunks of N5 lanes staged in shared memory; per-CTA FP64
-// partials are summed in a fixed order by k_wgrad_reduce.
-__global__ void __launch_bounds__(512) k_wgrad(const float* __restrict__ gout, int nout,
-                                               const float* __restrict__ in, int nin,
-                                               int64_t nchunks, int N5, int64_t fstride,
-                                               double* __restrict__ partial) {
-    extern __shared__ float sm[];
-    float* sg = sm;                              // [nout][4][N5] complex
-    float* sx = sm + (size_t)nout * 4 * N5 * 2;  // [nin][4][N5] complex
-    const int pairs = nout * nin;
-    const int t = threadIdx.x;
-    const int o = t / nin, i = t % nin;
-    float ar[4][4], ai[4][4];
+// Weight gradient of one parity: g[o][so][i][si] = sum_pixels gout[o][so]
+// conj(in[i][si]) over its (site, colour, lane) pixels, a [4 MF] x [4 NF]
+// complex product contracted over millions of pixels.
+//
+// Bound: the FP32 pipe (batch 4 at 16^4 x 12, even sites: 38.7 G
+// multiply-adds, 1.05 ms at 128 per clock and SM; its 3.6 GB of fields would
+// take half of that).  The fields hold pixels contiguously, the
+// product wants all rows of a pixel: 32 pixels at a time go through shared
+// memory transposed, [pixel][row], the in rows with both parts doubled
+// (xr, xr, xi, xi), so that a thread's 4 x 4 spin block of one (o, i) pair is
+// 32 paired multiply-adds (two per complex product: the pair (gr, gi) times
+// xr into A, times xi into B, combined once at the end) for 6 16-byte shared
+// loads.  A warp takes WO x WI pairs (4 x 8: its 32 in vectors are one
+// 128-byte row per load); the KS groups of warps take the pixels in turn; the
+// next 32 pixels are loaded into registers during the arithmetic.  One thread
+// per pair reading scalars from the fields' own order over both parities ran
+// at 7 TFLOP/s (29.8 ms each of the two gradients); the whole training step of
+// batch 4 at 16^4 x 12 went from 80.5 to 18.3 ms with this kernel and the
+// zero directions left out of the mixes.
+constexpr int kWgThreads = 256;
+constexpr int kWgPix = 32;
+
+template <int MF, int NF>
+struct WgShape {
+    static constexpr int WI = NF >= 8 ? 8 : 4, WO = 32 / WI;
+    static constexpr int WM = (MF + WO - 1) / WO, WN = (NF + WI - 1) / WI;
+    static constexpr int KS = (kWgThreads / 32) / (WM * WN);
+    static constexpr int GS = MF * 4 + 2;      // float2 per pixel row of gout
+    static constexpr int XS = NF * 4 + 1;      // float4 per pixel row of in
+    static constexpr size_t smem = kWgPix * ((size_t)GS * 8 + (size_t)XS * 16);
+    static_assert(WM * WN * KS * 32 == kWgThreads, "whole warps per pixel group");
+};
+
+template <int MF, int NF>
+__global__ void __launch_bounds__(kWgThreads, 2) k_wgrad(const float* __restrict__ gout,
+                                                         const float* __restrict__ in, int64_t npix, int N5,
+                                                         int64_t fstride, double* __restrict__ partial) {
+    using S = WgShape<MF, NF>;
+    constexpr int ROWS = 4 * (MF + NF);
+    constexpr int NLD = (ROWS + kWgThreads / 32 - 1) / (kWgThreads / 32);
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    float4* sx = reinterpret_cast<float4*>(sm_raw);                      // [pixel][si][i]
+    float2* sg = reinterpret_cast<float2*>(sx + (size_t)kWgPix * S::XS);   // [pixel][o][so]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ks = warp % S::KS, wt = warp / S::KS;
+    const int o = (wt / S::WN) * S::WO + lane / S::WI, i = (wt % S::WN) * S::WI + lane % S::WI;
+    const bool on = o < MF && i < NF;
+    const int oc = on ? o : 0, ic = on ? i : 0;      // idle lanes of a ragged shape compute on pair 0
+    float2 A[4][4], B[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) ar[a][b] = ai[a][b] = 0.f;
-    for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        const int64_t site = ch / 3;
-        const int colour = (int)(ch % 3);
-        __syncthreads();
-        const int ng = nout * 4 * N5, nx = nin * 4 * N5;
-        for (int e = t; e < ng + nx; e += blockDim.x) {
-            const bool isg = e < ng;
-            const int ee = isg ? e : e - ng;
-            const int fld = ee / (4 * N5), sp = (ee / N5) % 4, lane = ee % N5;
-            const float* src = (isg ? gout : in) + fld * fstride +
-                               2 * ((site * 12 + sp * 3 + colour) * N5 + lane);
-            const float2 v = *reinterpret_cast<const float2*>(src);
-            float* dst = (isg ? sg : sx) + 2 * ee;
-            dst[0] = v.x;
-            dst[1] = v.y;
+        for (int b = 0; b < 4; ++b) A[a][b] = B[a][b] = make_float2(0.f, 0.f);
+    float2 v[NLD];
+    auto load = [&](int64_t p0) {
+        const int64_t p = p0 + lane;
+        const bool live = p < npix;
+        const int64_t sc = live ? p / N5 : 0;
+        const int l = live ? (int)(p - sc * N5) : 0;
+        const int64_t site = sc / 3;
+        const int64_t base = (site * 12 + (sc - site * 3)) * N5 + l;
+#pragma unroll
+        for (int q = 0; q < NLD; ++q) {
+            const int row = warp + q * (kWgThreads / 32);
+            v[q] = make_float2(0.f, 0.f);
+            if (row < ROWS && live) {
+                const bool isg = row < 4 * MF;
+                const int rr = isg ? row : row - 4 * MF;
+                v[q] = *reinterpret_cast<const float2*>((isg ? gout : in) + (rr >> 2) * fstride +
+                                                        2 * (base + (int64_t)(rr & 3) * 3 * N5));
+            }
+        }
+    };
+    const int64_t step = (int64_t)gridDim.x * kWgPix;
+    int64_t p0 = (int64_t)blockIdx.x * kWgPix;
+    if (p0 < npix) load(p0);
+    for (; p0 < npix; p0 += step) {
+        __syncthreads();   // the previous pixels are no longer read
+#pragma unroll
+        for (int q = 0; q < NLD; ++q) {
+            const int row = warp + q * (kWgThreads / 32);
+            if (row < 4 * MF) sg[lane * S::GS + row] = v[q];
+            else if (row < ROWS) {
+                const int rr = row - 4 * MF;
+                sx[lane * S::XS + (rr & 3) * NF + (rr >> 2)] = make_float4(v[q].x, v[q].x, v[q].y, v[q].y);
+            }
         }
         __syncthreads();
-        if (t < pairs) {
-            for (int l = 0; l < N5; ++l) {
-                float gr[4], gi[4], xr[4], xi[4];
+        if (p0 + step < npix) load(p0 + step);
+#pragma unroll 2
+        for (int k = ks; k < kWgPix; k += S::KS) {
+            const float4* g4 = reinterpret_cast<const float4*>(sg + k * S::GS + oc * 4);
+            const float4 ga = g4[0], gb = g4[1];
+            const float2 g[4] = {make_float2(ga.x, ga.y), make_float2(ga.z, ga.w), make_float2(gb.x, gb.y),
+                                 make_float2(gb.z, gb.w)};
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const float4 x = sx[k * S::XS + b * NF + ic];
+                const float2 xr = make_float2(x.x, x.y), xi = make_float2(x.z, x.w);
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {
-                    gr[a] = sg[2 * ((o * 4 + a) * N5 + l)];
-                    gi[a] = sg[2 * ((o * 4 + a) * N5 + l) + 1];
-                    xr[a] = sx[2 * ((i * 4 + a) * N5 + l)];
-                    xi[a] = sx[2 * ((i * 4 + a) * N5 + l) + 1];
+                    A[a][b] = __ffma2_rn(g[a], xr, A[a][b]);
+                    B[a][b] = __ffma2_rn(g[a], xi, B[a][b]);
                 }
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {   // g_a * conj(x_b)
-                        ar[a][b] = fmaf(gr[a], xr[b], fmaf(gi[a], xi[b], ar[a][b]));
-                        ai[a][b] = fmaf(gi[a], xr[b], fmaf(-gr[a], xi[b], ai[a][b]));
-                    }
             }
         }
     }
-    if (t < pairs) {
-        double* out = partial + (size_t)blockIdx.x * pairs * 32;
+    if (on) {
+        double* out = partial + ((size_t)blockIdx.x * S::KS + ks) * (MF * NF * 32);
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
-                // layout [o][a][i][b] complex
-                const size_t idx = (((size_t)o * 4 + a) * nin + i) * 4 + b;
-                out[2 * idx] = (double)ar[a][b];
-                out[2 * idx + 1] = (double)ai[a][b];
+                const int idx = ((o * 4 + a) * NF + i) * 4 + b;   // g conj(x)
+                out[2 * idx] = (double)(A[a][b].x + B[a][b].y);
+                out[2 * idx + 1] = (double)(A[a][b].y - B[a][b].x);
             }
     }
 }
 
-__global__ void k_wgrad_reduce(const double* __restrict__ partial, int nblocks, int nval,
-                               double* __restrict__ out) {
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nval; v += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += partial[(size_t)b * nval + v];
-        out[v] = s;
-    }
+// Sum of the partials in a fixed order (8 slices, then the slices), written
+// in the master layout [d][channel][so][si]; dirs[j] is the direction of
+// field j on the side that runs over directions (gout for W2, in for W1).
+struct WgDirs { int d[8]; };
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const double* __restrict__ partial, int nparts, int mf, int nf,
+                                                      int C, bool dirs_out, WgDirs dirs, double* __restrict__ gw) {
+    __shared__ double sh[8][33];
+    const int nval = mf * nf * 32;
+    const int v = blockIdx.x * 32 + (threadIdx.x & 31), sl = threadIdx.x >> 5;
+    double s = 0.0;
+    if (v < nval)
+        for (int b = sl; b < nparts; b += 8) s += partial[(size_t)b * nval + v];
+    sh[sl][threadIdx.x & 31] = s;
+    __syncthreads();
+    if (sl != 0 || v >= nval) return;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) s += sh[q][threadIdx.x];
+    const int part = v & 1, si = (v >> 1) & 3, i = (v >> 3) % nf, oa = (v >> 3) / nf;
+    const int so = oa & 3, o = oa >> 2;
+    const int d = dirs.d[dirs_out ? o : i], ch = dirs_out ? i : o;
+    gw[2 * ((((size_t)d * C + ch) * 4 + so) * 4 + si) + part] = s;
 }
 
 // Adam on the real and imaginary parts (all arrays of n reals).
@@ -306,12 +377,14 @@ struct dwf_nn {
     float* d_w2 = nullptr;
     float* d_m = nullptr;    // Adam moments over [w1 | w2]
     float* d_v = nullptr;
-    float* d_mix1 = nullptr; // BF16-rounded mixing matrices, kernel layouts
-    float* d_mix2 = nullptr;
-    float* d_mix2h = nullptr;    // adjoint of layer-2 mixing
-    float* d_fold[2] = {nullptr, nullptr};   // W2 W1 on even / odd sites (inference)
+    // per parity, over that parity's directions: BF16-rounded mixing matrices in
+    // kernel layouts, the adjoint of layer 2, and W2 W1 (inference); one block
+    float* d_mix = nullptr;
+    float* mix1[2] = {nullptr, nullptr};
+    float* mix2[2] = {nullptr, nullptr};
+    float* mix2h[2] = {nullptr, nullptr};
+    float* fold[2] = {nullptr, nullptr};
     int adam_t = 0;
-    bool dirty = true;           // mixing matrices need a refresh
 };
 
 namespace dwf {
@@ -325,86 +398,102 @@ static size_t w2_len(int C) { return (size_t)kNDir * C * 16 * 2; }
 constexpr int kNFold[2] = {8, 3};
 constexpr int kFoldDirs[2][8] = {{1, 2, 3, 4, 5, 6, 7, 8}, {0, 9, 10, 0, 0, 0, 0, 0}};
 static size_t fold_len(int p) { return (size_t)kNFold[p] * 4 * kNFold[p] * 4 * 2; }
+static size_t mix_part_len(int C, int p) { return (size_t)kNFold[p] * C * 16 * 2; }
+static size_t mix_len(int C) {
+    size_t n = 0;
+    for (int p = 0; p < 2; ++p) n += 3 * mix_part_len(C, p) + fold_len(p);
+    return n;
+}
 
-static float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
+struct MixOut {
+    float* m1[2];
+    float* m2[2];
+    float* m2h[2];
+    float* fold[2];
+};
 
-// Rebuild the kernel-layout mixing matrices from the master weights (BF16 rounded).
-static dwf_status refresh_mix(dwf_nn* K) {
-    if (!K->dirty) return DWF_OK;
-    const int C = K->C;
-    std::vector<float> w1(w1_len(C)), w2(w2_len(C));
-    DWF_CUDA(cudaMemcpy(w1.data(), K->d_w1, w1.size() * 4, cudaMemcpyDeviceToHost));
-    DWF_CUDA(cudaMemcpy(w2.data(), K->d_w2, w2.size() * 4, cudaMemcpyDeviceToHost));
-    // mix1: [o = a][so][i = d][si]  <- W1[d][a][so][si]
-    std::vector<float> m1((size_t)C * 4 * kNDir * 4 * 2), m2((size_t)kNDir * 4 * C * 4 * 2),
-        m2h((size_t)C * 4 * kNDir * 4 * 2);
-    for (int d = 0; d < kNDir; ++d)
-        for (int a = 0; a < C; ++a)
-            for (int so = 0; so < 4; ++so)
-                for (int si = 0; si < 4; ++si) {
-                    const size_t src1 = (((size_t)d * C + a) * 4 + so) * 4 + si;
-                    const size_t dst1 = (((size_t)a * 4 + so) * kNDir + d) * 4 + si;
-                    m1[2 * dst1] = bf16_round(w1[2 * src1]);
-                    m1[2 * dst1 + 1] = bf16_round(w1[2 * src1 + 1]);
-                    // W2[d][0][b = a][so][si] -> mix2 [o = d][so][i = b][si]
-                    const size_t dst2 = (((size_t)d * 4 + so) * C + a) * 4 + si;
-                    const float r2 = bf16_round(w2[2 * src1]), i2 = bf16_round(w2[2 * src1 + 1]);
-                    m2[2 * dst2] = r2;
-                    m2[2 * dst2 + 1] = i2;
-                    // adjoint: g_phi[b][si] = sum_{d,so} conj(W2[d][b][so][si]) g_psi[d][so]
-                    //   -> mix2h [o = b][so' = si][i = d][si' = so] = conj(W2[d][b][so][si])
-                    const size_t dsth = (((size_t)a * 4 + si) * kNDir + d) * 4 + so;
-                    m2h[2 * dsth] = r2;
-                    m2h[2 * dsth + 1] = -i2;
+__device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
+
+// Mixing matrices from the FP32 master weights (rounded to BF16), per parity p
+// over its n directions d = dirs[p][.]:
+//   m1  [o = a][so][i = d][si]  = W1[d][a][so][si]
+//   m2  [o = d][so][i = b][si]  = W2[d][b][so][si]
+//   m2h [o = b][so][i = d][si]  = conj(W2[d][b][si][so])
+//   fold[o = d][so][i = d'][si] = sum_{b,t} W2[d][b][so][t] W1[d'][b][t][si]
+// (fold: FP64 products, stored FP32).  One thread per complex entry.
+struct MixDirs { int n[2]; int d[2][8]; };
+__global__ void k_mix_weights(const float* __restrict__ w1, const float* __restrict__ w2, int C, MixDirs md, MixOut out) {
+    const int p = blockIdx.y, n = md.n[p];
+    const int nw = n * C * 16, nf = n * n * 16;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nw + nf; e += gridDim.x * blockDim.x) {
+        if (e < nw) {
+            const int si = e & 3, so = (e >> 2) & 3, ch = (e >> 4) % C, j = (e >> 4) / C;
+            const size_t src = (((size_t)md.d[p][j] * C + ch) * 4 + so) * 4 + si;
+            const float r2 = bf16_round(w2[2 * src]), i2 = bf16_round(w2[2 * src + 1]);
+            const size_t o1 = (((size_t)ch * 4 + so) * n + j) * 4 + si, o2 = (((size_t)j * 4 + so) * C + ch) * 4 + si,
+                         oh = (((size_t)ch * 4 + si) * n + j) * 4 + so;
+            out.m1[p][2 * o1] = bf16_round(w1[2 * src]);
+            out.m1[p][2 * o1 + 1] = bf16_round(w1[2 * src + 1]);
+            out.m2[p][2 * o2] = r2;
+            out.m2[p][2 * o2 + 1] = i2;
+            out.m2h[p][2 * oh] = r2;
+            out.m2h[p][2 * oh + 1] = -i2;
+        } else {
+            const int f = e - nw;
+            const int si = f & 3, so = (f >> 2) & 3, i = (f >> 4) % n, o = (f >> 4) / n;
+            double mr = 0.0, mi = 0.0;
+            for (int b = 0; b < C; ++b)
+                for (int t = 0; t < 4; ++t) {
+                    const size_t q2 = (((size_t)md.d[p][o] * C + b) * 4 + so) * 4 + t;
+                    const size_t q1 = (((size_t)md.d[p][i] * C + b) * 4 + t) * 4 + si;
+                    const double ar = bf16_round(w2[2 * q2]), ai = bf16_round(w2[2 * q2 + 1]);
+                    const double br = bf16_round(w1[2 * q1]), bi = bf16_round(w1[2 * q1 + 1]);
+                    mr += ar * br - ai * bi;
+                    mi += ar * bi + ai * br;
                 }
-    DWF_CUDA(cudaMemcpy(K->d_mix1, m1.data(), m1.size() * 4, cudaMemcpyHostToDevice));
-    DWF_CUDA(cudaMemcpy(K->d_mix2, m2.data(), m2.size() * 4, cudaMemcpyHostToDevice));
-    DWF_CUDA(cudaMemcpy(K->d_mix2h, m2h.data(), m2h.size() * 4, cudaMemcpyHostToDevice));
-    // folded layers for inference: M[d][d'] = sum_b W2[d][b] W1[d'][b] (4x4 complex
-    // spin blocks, FP64 products of the BF16-rounded weights, stored FP32) in the
-    // mixing layout [o = d][so][i = d'][si], restricted to each parity's directions
-    for (int p = 0; p < 2; ++p) {
-        const int n = kNFold[p];
-        std::vector<float> fm(fold_len(p));
-        for (int o = 0; o < n; ++o)
-            for (int i = 0; i < n; ++i)
-                for (int so = 0; so < 4; ++so)
-                    for (int si = 0; si < 4; ++si) {
-                        const int d = kFoldDirs[p][o], dp = kFoldDirs[p][i];
-                        double mr = 0.0, mi = 0.0;
-                        for (int b = 0; b < C; ++b)
-                            for (int t = 0; t < 4; ++t) {
-                                const size_t i2 = (((size_t)d * C + b) * 4 + so) * 4 + t;
-                                const size_t i1 = (((size_t)dp * C + b) * 4 + t) * 4 + si;
-                                const double ar = bf16_round(w2[2 * i2]), ai = bf16_round(w2[2 * i2 + 1]);
-                                const double br = bf16_round(w1[2 * i1]), bi = bf16_round(w1[2 * i1 + 1]);
-                                mr += ar * br - ai * bi;
-                                mi += ar * bi + ai * br;
-                            }
-                        const size_t dst = (((size_t)o * 4 + so) * n + i) * 4 + si;
-                        fm[2 * dst] = (float)mr;
-                        fm[2 * dst + 1] = (float)mi;
-                    }
-        DWF_CUDA(cudaMemcpy(K->d_fold[p], fm.data(), fm.size() * 4, cudaMemcpyHostToDevice));
+            const size_t dst = (((size_t)o * 4 + so) * n + i) * 4 + si;
+            out.fold[p][2 * dst] = (float)mr;
+            out.fold[p][2 * dst + 1] = (float)mi;
+        }
     }
-    K->dirty = false;
+}
+
+// Rebuild the mixing matrices after the master weights changed, on stream s;
+// every caller waits for s before it returns, so that a later call may use
+// them on any stream.
+static dwf_status refresh_mix(dwf_nn* K, cudaStream_t s) {
+    MixDirs md{};
+    MixOut mo{};
+    for (int p = 0; p < 2; ++p) {
+        md.n[p] = kNFold[p];
+        for (int j = 0; j < kNFold[p]; ++j) md.d[p][j] = kFoldDirs[p][j];
+        mo.m1[p] = K->mix1[p];
+        mo.m2[p] = K->mix2[p];
+        mo.m2h[p] = K->mix2h[p];
+        mo.fold[p] = K->fold[p];
+    }
+    k_mix_weights<<<dim3(12, 2), 256, 0, s>>>(K->d_w1, K->d_w2, K->C, md, mo);
+    note_launch();
+    DWF_CUDA(cudaGetLastError());
     return DWF_OK;
 }
 
-// network workspace of a handle for nrhs lanes
+// network workspace of a handle for nrhs lanes.  Field j of R, psi on parity p
+// belongs to direction kFoldDirs[p][j]: what is exactly zero (below) has no
+// storage.
 struct NNWS {
     int nrhs = 0, C = 0;
-    float* x0 = nullptr;      // embedded input (full field)
-    float* R = nullptr;       // 11 full fields
-    float* phi = nullptr;     // C full fields
-    float* psi = nullptr;     // 11 full fields
-    float* z = nullptr;       // full field
+    float* R = nullptr;       // 8 full fields
+    float* psi = nullptr;     // 8 full fields
+    float* phi = nullptr;     // C full fields (training)
     float* gphi = nullptr;    // C full fields (training)
+    float* z = nullptr;       // odd FP32 fields (training): K r, then the gradient of the loss
     float* at = nullptr;      // odd FP32 temporaries for the energy-norm loss
     float* aw = nullptr;
     double* wpart = nullptr;  // weight-gradient partials
-    double* gw = nullptr;     // [gW1 | gW2]
-    int wblocks = 0;
+    double* gw = nullptr;     // [gW1 | gW2], master layout
+    double* scal = nullptr;   // loss scalars [4][nrhs]
+    double* part = nullptr;   // loss partials (per tile and right-hand side)
 };
 
 static std::map<dwf_handle*, NNWS> g_nnws;
@@ -413,26 +502,47 @@ static int64_t full_floats(const dwf_handle* h, int nrhs) {
     return (int64_t)(h->nsite[0] + h->nsite[1]) * 12 * h->p.Ls * nrhs * 2;
 }
 
+static void free_nn_bufs(NNWS& w) {
+    void* p[] = {w.R, w.psi, w.phi, w.gphi, w.z, w.at, w.aw, w.wpart, w.gw, w.scal, w.part};
+    for (void* q : p) cudaFree(q);
+    w = NNWS();
+}
+
+constexpr int kWgBlocks = 152 * 2;
+constexpr int kMaxTrainLanes = 236;   // Ls * nrhs of a training batch (Ls is even)
+
+template <int MF, int NF>
+static cudaError_t wgrad_attr() {
+    return cudaFuncSetAttribute(k_wgrad<MF, NF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)WgShape<MF, NF>::smem);
+}
+
 static dwf_status nn_ws(dwf_handle* h, int nrhs, int C, bool train, NNWS** out) {
     NNWS& w = g_nnws[h];
     if (w.nrhs != nrhs || w.C != C || (train && w.gphi == nullptr)) {
-        cudaFree(w.x0); cudaFree(w.R); cudaFree(w.phi); cudaFree(w.psi); cudaFree(w.z);
-        cudaFree(w.gphi); cudaFree(w.wpart); cudaFree(w.gw); cudaFree(w.at); cudaFree(w.aw);
-        w = NNWS();
+        free_nn_bufs(w);
         const int64_t f = full_floats(h, nrhs);
-        DWF_CUDA(dev_malloc(&w.x0, f * 4));
-        DWF_CUDA(dev_malloc(&w.R, (size_t)kNDir * f * 4));
-        DWF_CUDA(dev_malloc(&w.phi, (size_t)C * f * 4));
-        DWF_CUDA(dev_malloc(&w.psi, (size_t)kNDir * f * 4));
-        DWF_CUDA(dev_malloc(&w.z, f * 4));
         if (train) {
-            DWF_CUDA(dev_malloc(&w.gphi, (size_t)C * f * 4));
-            w.wblocks = 152 * 2;
-            DWF_CUDA(dev_malloc(&w.wpart, (size_t)w.wblocks * C * kNDir * 32 * sizeof(double)));
+            DWF_CUDA((wgrad_attr<kNFold[0], 16>()));
+            DWF_CUDA((wgrad_attr<16, kNFold[0]>()));
+            DWF_CUDA((wgrad_attr<kNFold[1], 16>()));
+            DWF_CUDA((wgrad_attr<16, kNFold[1]>()));
+        }
+        DWF_CUDA(dev_malloc(&w.R, (size_t)kNFold[0] * f * 4));
+        DWF_CUDA(dev_malloc(&w.psi, (size_t)kNFold[0] * f * 4));
+        if (train) {
+            DWF_CUDA(dev_malloc(&w.phi, (size_t)C * f * 4));
+            const size_t pairs8 = (size_t)kWgBlocks * WgShape<8, 16>::KS * 8 * 16 * 32;
+            const size_t pairs3 = (size_t)kWgBlocks * WgShape<3, 16>::KS * 3 * 16 * 32;
+            DWF_CUDA(dev_malloc(&w.wpart, std::max(pairs8, pairs3) * sizeof(double)));
             DWF_CUDA(dev_malloc(&w.gw, (w1_len(C) + w2_len(C)) * sizeof(double)));
             const size_t odd = (size_t)h->nsite[1] * 12 * h->p.Ls * nrhs * 2;
+            DWF_CUDA(dev_malloc(&w.z, odd * 4));
             DWF_CUDA(dev_malloc(&w.at, odd * 4));
             DWF_CUDA(dev_malloc(&w.aw, odd * 4));
+            DWF_CUDA(dev_malloc(&w.scal, (size_t)4 * nrhs * sizeof(double)));
+            DWF_CUDA(dev_malloc(&w.part, (size_t)(h->nsite[1] / kMinTile + h->nbox + 1) * nrhs * sizeof(double)));
+            DWF_CUDA(dev_malloc(&w.gphi, (size_t)C * f * 4));
         }
         w.nrhs = nrhs;
         w.C = C;
@@ -444,55 +554,43 @@ static dwf_status nn_ws(dwf_handle* h, int nrhs, int C, bool train, NNWS** out) 
 void free_nn_ws(dwf_handle* h) {
     auto it = g_nnws.find(h);
     if (it == g_nnws.end()) return;
-    NNWS& w = it->second;
-    cudaFree(w.x0); cudaFree(w.R); cudaFree(w.phi); cudaFree(w.psi); cudaFree(w.z);
-    cudaFree(w.gphi); cudaFree(w.wpart); cudaFree(w.gw); cudaFree(w.at); cudaFree(w.aw);
+    free_nn_bufs(it->second);
     g_nnws.erase(it);
 }
 
-static TransArgs trans_args(dwf_handle* h, int nrhs, int p) {
-    TransArgs a{};
-    a.N5 = h->p.Ls * nrhs;
-    a.Ls = h->p.Ls;
-    a.parity = p;
-    const int64_t c0 = h->nsite[0] * 12 * (int64_t)a.N5 * 2;
-    a.off_p = p ? c0 : 0;
-    a.off_q = p ? 0 : c0;
-    a.fstride = full_floats(h, nrhs);
-    a.links = (const float*)h->d_links[DWF_FP32][p];
-    a.nbr = h->d_nbr[p];
-    return a;
-}
-
-static dwf_status launch_transport(dwf_handle* h, int nrhs, const float* in, float* out,
-                                   const int* dirs, int ndir, bool sum, const float* const* ins,
-                                   cudaStream_t s, int only_parity = -1) {
+// T_{dirs[j]} of one field into fields out + j ostride (multi), or the sum of
+// T_{dirs[j]} of the input fields (sum), on the sites of parity p.  same / opp
+// are the input's blocks of parity p and 1 - p.
+static dwf_status launch_transport(dwf_handle* h, int nrhs, int p, const float* same, const float* opp, float* out,
+                                   const int* dirs, int ndir, bool sum, cudaStream_t s) {
     const TileSet* tsp = nullptr;
     DWF_TRY(get_tiles(h, tile_for(h, nrhs), &tsp));
     const TileSet& ts = *tsp;
-    for (int p = 0; p < 2; ++p) {
-        if (ts.ntiles[p] == 0 || (only_parity >= 0 && p != only_parity)) continue;
-        TransArgs a = trans_args(h, nrhs, p);
-        a.in = in;
-        a.out = out;
-        a.ins = ins;
-        a.tiles = ts.d_tiles[p];
-        a.ndir = ndir;
-        for (int j = 0; j < ndir; ++j) a.dirs[j] = dirs[j];
-        if (sum) k_transport_sum<<<ts.ntiles[p], 256, 0, s>>>(a);
-        else k_transport_multi<<<ts.ntiles[p], 256, 0, s>>>(a);
-        note_launch();
-        DWF_CUDA(cudaGetLastError());
-    }
+    if (ts.ntiles[p] == 0) return DWF_OK;
+    TransArgs a{};
+    a.same = same;
+    a.opp = opp;
+    a.out = out;
+    a.links = (const float*)h->d_links[DWF_FP32][p];
+    a.nbr = h->d_nbr[p];
+    a.tiles = ts.d_tiles[p];
+    a.N5 = h->p.Ls * nrhs;
+    a.Ls = h->p.Ls;
+    a.istride = a.ostride = full_floats(h, nrhs);
+    a.ndir = ndir;
+    for (int j = 0; j < ndir; ++j) a.dirs[j] = dirs[j];
+    if (sum) k_transport_sum<<<ts.ntiles[p], 256, 0, s>>>(a);
+    else k_transport_multi<<<ts.ntiles[p], 256, 0, s>>>(a);
+    note_launch();
+    DWF_CUDA(cudaGetLastError());
     return DWF_OK;
 }
 
-// Mixing on a full field, or (parity 0 / 1) on that parity's block only: `in`
-// and `out` then point at the block, fields keep the full-field stride.
-static dwf_status launch_mix(dwf_handle* h, int nrhs, const float* in, int nin, float* out, int nout,
-                             const float* W, cudaStream_t s, int only_parity = -1) {
-    const int64_t nsites = only_parity < 0 ? h->nsite[0] + h->nsite[1] : h->nsite[only_parity];
-    const int64_t npix = nsites * 3 * (int64_t)h->p.Ls * nrhs;
+// Mixing on the block of parity p (`in` and `out` point at the block, fields
+// keep the full-field stride).
+static dwf_status launch_mix(dwf_handle* h, int nrhs, int p, const float* in, int nin, float* out, int nout,
+                             const float* W, cudaStream_t s) {
+    const int64_t npix = h->nsite[p] * 3 * (int64_t)h->p.Ls * nrhs;
     if (npix == 0) return DWF_OK;
     const int64_t fstride = full_floats(h, nrhs);
     const size_t smem = (size_t)nout * 4 * nin * 4 * 2 * sizeof(float);
@@ -501,8 +599,6 @@ static dwf_status launch_mix(dwf_handle* h, int nrhs, const float* in, int nin, 
     const int N5 = h->p.Ls * nrhs;
     if (nout == 16)
         k_mix<16><<<(int)blocks, 128, smem, s>>>(in, nin, out, W, npix, N5, fstride);
-    else if (nout == 11)
-        k_mix<11><<<(int)blocks, 128, smem, s>>>(in, nin, out, W, npix, N5, fstride);
     else if (nout == 8)
         k_mix<8><<<(int)blocks, 128, smem, s>>>(in, nin, out, W, npix, N5, fstride);
     else if (nout == 3)
@@ -516,88 +612,70 @@ static dwf_status launch_mix(dwf_handle* h, int nrhs, const float* in, int nin, 
     return DWF_OK;
 }
 
-static dwf_status launch_wgrad(dwf_handle* h, NNWS& w, int nrhs, const float* gout, int nout,
-                               const float* in, int nin, double* dst, cudaStream_t s) {
+// gW of one layer from parity p's pixels: MF fields of gout against NF of in;
+// dirs_out: the gout side runs over directions (W2), else the in side (W1).
+template <int MF, int NF>
+static dwf_status launch_wgrad(dwf_handle* h, NNWS& w, int nrhs, int p, const float* gout, const float* in,
+                               bool dirs_out, double* dst, cudaStream_t s) {
+    using S = WgShape<MF, NF>;
     const int N5 = h->p.Ls * nrhs;
-    const int64_t nchunks = (h->nsite[0] + h->nsite[1]) * 3;
-    const int64_t fstride = full_floats(h, nrhs);
-    int threads = (nout * nin + 31) / 32 * 32;
-    const size_t smem = (size_t)(nout + nin) * 4 * N5 * 2 * sizeof(float);
-    static bool attr = false;
-    if (!attr) {
-        DWF_CUDA(cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-        attr = true;
-    }
-    if (smem > 200 * 1024) {
-        set_error("nn: %d lanes need %zu bytes of shared memory for the weight gradient", N5, smem);
-        return DWF_ERR_UNSUPPORTED;
-    }
-    k_wgrad<<<w.wblocks, threads, smem, s>>>(gout, nout, in, nin, nchunks, N5, fstride, w.wpart);
+    const int64_t npix = h->nsite[p] * 3 * (int64_t)N5;
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((npix + kWgPix - 1) / kWgPix, kWgBlocks));
+    k_wgrad<MF, NF><<<blocks, kWgThreads, S::smem, s>>>(gout, in, npix, N5, full_floats(h, nrhs), w.wpart);
     note_launch();
     DWF_CUDA(cudaGetLastError());
-    const int nval = nout * nin * 32;
-    k_wgrad_reduce<<<(nval + 255) / 256, 256, 0, s>>>(w.wpart, w.wblocks, nval, dst);
+    WgDirs wd{};
+    for (int j = 0; j < kNFold[p]; ++j) wd.d[j] = kFoldDirs[p][j];
+    constexpr int nval = MF * NF * 32;
+    k_wgrad_reduce<<<nval / 32, 256, 0, s>>>(w.wpart, blocks * S::KS, MF, NF, w.C, dirs_out, wd, dst);
     note_launch();
     DWF_CUDA(cudaGetLastError());
     return DWF_OK;
 }
 
-static const int kDirsFwd[kNDir] = {0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10};
-
-// z = K x0 (x0 full field with the input on odd sites, zero on even)
-static dwf_status nn_forward(dwf_nn* K, dwf_handle* h, NNWS& w, int nrhs, cudaStream_t s) {
-    const int C = K->C;
-    DWF_TRY(refresh_mix(K));
-    DWF_TRY(launch_transport(h, nrhs, w.x0, w.R, kDirsFwd, kNDir, false, nullptr, s));
-    DWF_TRY(launch_mix(h, nrhs, w.R, kNDir, w.phi, C, K->d_mix1, s));
-    DWF_TRY(launch_mix(h, nrhs, w.phi, C, w.psi, kNDir, K->d_mix2, s));
-    const int64_t f = full_floats(h, nrhs);
-    const float* ins[kNDir];
-    for (int d = 0; d < kNDir; ++d) ins[d] = w.psi + d * f;
-    // device array of pointers
-    static thread_local const float** d_ins = nullptr;
-    if (d_ins == nullptr) DWF_CUDA(dev_malloc(&d_ins, kNDir * sizeof(float*)));
-    DWF_CUDA(cudaMemcpyAsync(d_ins, ins, sizeof(ins), cudaMemcpyHostToDevice, s));
-    return launch_transport(h, nrhs, nullptr, w.z, kDirsFwd, kNDir, true, d_ins, s);
+// z = sum_d T_d psi_d on odd sites; psi's field j on parity p holds direction
+// kFoldDirs[p][j]
+static dwf_status psi_sum(dwf_handle* h, int nrhs, const float* psi, float* z, cudaStream_t s) {
+    int dirs[kNDir], nd = 0;
+    for (int p = 1; p >= 0; --p)
+        for (int j = 0; j < kNFold[p]; ++j) dirs[nd++] = kFoldDirs[p][j];
+    const int64_t c0 = h->nsite[0] * 12 * (int64_t)h->p.Ls * nrhs * 2;
+    return launch_transport(h, nrhs, 1, psi + c0, psi, z, dirs, nd, true, s);
 }
 
-// Inference z = K x on the odd checkerboard.  The same function as
-// nn_forward up to rounding, with the work that is exactly zero left out: x0
-// vanishes on even sites, so R_d = T_d x0 is zero on odd sites for the link
-// directions 1..8 and on even sites for 0, 9 and 10; only odd z is read, which
-// takes psi_d on even sites for d = 1..8 and on odd sites for 0, 9, 10; and
-// with no nonlinearity between the layers psi = (W2 W1) R.  Per parity the
-// folded 4x4-block matrix over that parity's directions (8 x 8 blocks even,
-// 3 x 3 odd) replaces the two mixes through the C channels.
+// z = K x on the odd checkerboard through the channels (training: R and phi
+// are kept for the gradient).  What is exactly zero is left out throughout:
+// x vanishes on even sites, so R_d = T_d x is zero on odd sites for the link
+// directions 1..8 and on even sites for 0, 9 and 10; z is read on odd sites
+// only, which take psi_d from even sites for d = 1..8 and from odd sites for
+// 0, 9, 10.
+static dwf_status nn_forward(dwf_nn* K, dwf_handle* h, NNWS& w, const float* x, int nrhs, cudaStream_t s) {
+    const int64_t c0 = h->nsite[0] * 12 * (int64_t)h->p.Ls * nrhs * 2;
+    for (int p = 0; p < 2; ++p) {
+        const int64_t o = p ? c0 : 0;
+        const int n = kNFold[p];
+        DWF_TRY(launch_transport(h, nrhs, p, x, x, w.R + o, kFoldDirs[p], n, false, s));
+        DWF_TRY(launch_mix(h, nrhs, p, w.R + o, n, w.phi + o, K->C, K->mix1[p], s));
+        DWF_TRY(launch_mix(h, nrhs, p, w.phi + o, K->C, w.psi + o, n, K->mix2[p], s));
+    }
+    return psi_sum(h, nrhs, w.psi, w.z, s);
+}
+
+// Inference z = K x on the odd checkerboard: the same function as nn_forward
+// up to rounding; with no nonlinearity between the layers psi = (W2 W1) R, so
+// per parity the folded 4x4-block matrix over that parity's directions (8 x 8
+// blocks even, 3 x 3 odd) replaces the two mixes through the C channels.
 dwf_status nn_apply_internal(dwf_nn* K, dwf_handle* h, float* out, const float* in, int nrhs,
                              cudaStream_t s) {
     NNWS* w;
     DWF_TRY(nn_ws(h, nrhs, K->C, false, &w));
-    DWF_TRY(refresh_mix(K));
     const int64_t c0 = h->nsite[0] * 12 * (int64_t)h->p.Ls * nrhs * 2;
-    const int64_t c1 = h->nsite[1] * 12 * (int64_t)h->p.Ls * nrhs * 2;
-    const int64_t f = full_floats(h, nrhs);
-    // the even block of x0 is never read below
-    DWF_CUDA(cudaMemcpyAsync(w->x0 + c0, in, c1 * 4, cudaMemcpyDeviceToDevice, s));
-    for (int p = 0; p < 2; ++p)
-        DWF_TRY(launch_transport(h, nrhs, w->x0, w->R, kFoldDirs[p], kNFold[p], false, nullptr, s, p));
-    DWF_TRY(launch_mix(h, nrhs, w->R, kNFold[0], w->psi, kNFold[0], K->d_fold[0], s, 0));
-    DWF_TRY(launch_mix(h, nrhs, w->R + c0, kNFold[1], w->psi + c0, kNFold[1], K->d_fold[1], s, 1));
-    // z on odd sites: psi field j holds direction kFoldDirs[p][j] on parity p
-    int dirs[kNDir];
-    const float* ins[kNDir];
-    int nd = 0;
-    for (int p = 1; p >= 0; --p)
-        for (int j = 0; j < kNFold[p]; ++j) {
-            dirs[nd] = kFoldDirs[p][j];
-            ins[nd++] = w->psi + j * f;
-        }
-    static thread_local const float** d_ins = nullptr;
-    if (d_ins == nullptr) DWF_CUDA(dev_malloc(&d_ins, kNDir * sizeof(float*)));
-    DWF_CUDA(cudaMemcpyAsync(d_ins, ins, sizeof(ins), cudaMemcpyHostToDevice, s));
-    DWF_TRY(launch_transport(h, nrhs, nullptr, w->z, dirs, kNDir, true, d_ins, s, 1));
-    DWF_CUDA(cudaMemcpyAsync(out, w->z + c0, c1 * 4, cudaMemcpyDeviceToDevice, s));
-    return DWF_OK;
+    for (int p = 0; p < 2; ++p) {
+        const int64_t o = p ? c0 : 0;
+        DWF_TRY(launch_transport(h, nrhs, p, in, in, w->R + o, kFoldDirs[p], kNFold[p], false, s));
+        DWF_TRY(launch_mix(h, nrhs, p, w->R + o, kNFold[p], w->psi + o, kNFold[p], K->fold[p], s));
+    }
+    return psi_sum(h, nrhs, w->psi, out, s);
 }
 
 }  // namespace dwf
@@ -622,18 +700,26 @@ dwf_status dwf_nn_create(dwf_nn** out, int channels) {
     if (dev_malloc(&K->d_w1, n1 * 4) != cudaSuccess || dev_malloc(&K->d_w2, n2 * 4) != cudaSuccess ||
         dev_malloc(&K->d_m, (n1 + n2) * 4) != cudaSuccess ||
         dev_malloc(&K->d_v, (n1 + n2) * 4) != cudaSuccess ||
-        dev_malloc(&K->d_mix1, n1 * 4) != cudaSuccess || dev_malloc(&K->d_mix2, n2 * 4) != cudaSuccess ||
-        dev_malloc(&K->d_mix2h, n2 * 4) != cudaSuccess ||
-        dev_malloc(&K->d_fold[0], fold_len(0) * 4) != cudaSuccess ||
-        dev_malloc(&K->d_fold[1], fold_len(1) * 4) != cudaSuccess) {
+        dev_malloc(&K->d_mix, mix_len(channels) * 4) != cudaSuccess) {
         set_error("dwf_nn_create: cudaMalloc failed");
+        dwf_nn_destroy(K);
         return DWF_ERR_CUDA;
+    }
+    float* m = K->d_mix;
+    for (int p = 0; p < 2; ++p) {
+        float** part[3] = {&K->mix1[p], &K->mix2[p], &K->mix2h[p]};
+        for (float** q : part) { *q = m; m += mix_part_len(channels, p); }
+        K->fold[p] = m;
+        m += fold_len(p);
     }
     cudaMemcpy(K->d_w1, K->w1.data(), n1 * 4, cudaMemcpyHostToDevice);
     cudaMemcpy(K->d_w2, K->w2.data(), n2 * 4, cudaMemcpyHostToDevice);
     cudaMemset(K->d_m, 0, (n1 + n2) * 4);
     cudaMemset(K->d_v, 0, (n1 + n2) * 4);
-    K->dirty = true;
+    if (refresh_mix(K, nullptr) != DWF_OK || cudaStreamSynchronize(nullptr) != cudaSuccess) {
+        dwf_nn_destroy(K);
+        return DWF_ERR_CUDA;
+    }
     *out = K;
     return DWF_OK;
 }
@@ -641,8 +727,7 @@ dwf_status dwf_nn_create(dwf_nn** out, int channels) {
 dwf_status dwf_nn_destroy(dwf_nn* K) {
     if (!K) return DWF_OK;
     cudaFree(K->d_w1); cudaFree(K->d_w2); cudaFree(K->d_m); cudaFree(K->d_v);
-    cudaFree(K->d_mix1); cudaFree(K->d_mix2); cudaFree(K->d_mix2h);
-    cudaFree(K->d_fold[0]); cudaFree(K->d_fold[1]);
+    cudaFree(K->d_mix);
     delete K;
     return DWF_OK;
 }
@@ -658,7 +743,8 @@ dwf_status dwf_nn_set_weights(dwf_nn* K, const double* w, size_t n) {
     for (size_t i = 0; i < 2 * n; ++i) all[i] = (float)w[i];
     DWF_CUDA(cudaMemcpy(K->d_w1, all.data(), n1 * 4, cudaMemcpyHostToDevice));
     DWF_CUDA(cudaMemcpy(K->d_w2, all.data() + n1, (2 * n - n1) * 4, cudaMemcpyHostToDevice));
-    K->dirty = true;
+    DWF_TRY(refresh_mix(K, nullptr));
+    DWF_CUDA(cudaStreamSynchronize(nullptr));
     return DWF_OK;
 }
 
@@ -802,29 +888,25 @@ dwf_status dwf_nn_train_step(dwf_nn* K, dwf_handle* h, const float* r, const flo
         return DWF_ERR_ARG;
     }
     cudaStream_t s = (cudaStream_t)stream;
+    if (h->p.Ls * nrhs > kMaxTrainLanes) {
+        set_error("nn: %d lanes exceed the training step's %d", h->p.Ls * nrhs, kMaxTrainLanes);
+        return DWF_ERR_UNSUPPORTED;
+    }
     NNWS* wp;
     DWF_TRY(nn_ws(h, nrhs, K->C, true, &wp));
     NNWS& w = *wp;
     const int C = K->C;
     const int64_t c0 = h->nsite[0] * 12 * (int64_t)h->p.Ls * nrhs * 2;
     const int64_t c1 = h->nsite[1] * 12 * (int64_t)h->p.Ls * nrhs * 2;
-    const int64_t f = full_floats(h, nrhs);
-    DWF_CUDA(cudaMemsetAsync(w.x0, 0, c0 * 4, s));
-    DWF_CUDA(cudaMemcpyAsync(w.x0 + c0, r, c1 * 4, cudaMemcpyDeviceToDevice, s));
-    DWF_TRY(nn_forward(K, h, w, nrhs, s));
+    DWF_TRY(nn_forward(K, h, w, r, nrhs, s));
     const int T = tile_for(h, nrhs);
-    const TileSet* tsp = nullptr;
-    DWF_TRY(get_tiles(h, T, &tsp));
-    const TileSet& ts = *tsp;
     std::vector<double> h1(nrhs), h2(nrhs), h3(nrhs);
-    double* d_scal;
-    DWF_CUDA(dev_malloc(&d_scal, (size_t)(4 * nrhs + (ts.ntiles[1] + 1) * nrhs) * sizeof(double)));
-    double* d1 = d_scal;
-    double* d2 = d_scal + nrhs;
-    double* d_coef = d_scal + 2 * nrhs;
-    double* d3 = d_scal + 3 * nrhs;
-    double* part = d_scal + 4 * nrhs;
-    float* zo = w.z + c0;
+    double* d1 = w.scal;
+    double* d2 = w.scal + nrhs;
+    double* d_coef = w.scal + 2 * nrhs;
+    double* d3 = w.scal + 3 * nrhs;
+    double* part = w.part;
+    float* zo = w.z;
     auto dot = [&](const void* x, const void* y, double* dst) -> dwf_status {
         DWF_TRY(launch_dot_partial(h, 1, x, y, DWF_FP32, DWF_FP32, nrhs, part, T, s));
         return launch_reduce_sys(h, 1, part, nrhs, dst, T, s);
@@ -880,35 +962,27 @@ dwf_status dwf_nn_train_step(dwf_nn* K, dwf_handle* h, const float* r, const flo
     }
     if (loss) *loss = L;
     DWF_CUDA(cudaMemcpyAsync(d_coef, coef.data(), nrhs * 8, cudaMemcpyHostToDevice, s));
-    // g_z = coef * (held residual) on odd sites, zero on even sites
-    DWF_CUDA(cudaMemsetAsync(w.z, 0, c0 * 4, s));
+    // g_z = coef * (held residual) on odd sites (zero on even sites, so the same
+    // directions survive per parity as in the forward pass)
     DWF_TRY(launch_axpby(h, 1, nrhs, nullptr, 0.0, nullptr, DWF_FP32, d_coef, 0.0, zo, DWF_FP32, nullptr, T, s));
-    // g_psi_d = T_d^+ g_z  (into psi)
-    DWF_TRY(launch_transport(h, nrhs, w.z, w.psi, kAdj, kNDir, false, nullptr, s));
-    // gW2[o = d][so][i = b][si] = sum g_psi_d phi_b^+
-    DWF_TRY(launch_wgrad(h, w, nrhs, w.psi, kNDir, w.phi, C, w.gw + w1_len(C), s));
-    // g_phi = W2^+ g_psi
-    DWF_TRY(launch_mix(h, nrhs, w.psi, kNDir, w.gphi, C, K->d_mix2h, s));
-    // gW1[o = a][so][i = d][si] = sum g_phi_a R_d^+
-    DWF_TRY(launch_wgrad(h, w, nrhs, w.gphi, C, w.R, kNDir, w.gw, s));
-    // gradients are in kernel layouts: convert to the master (oracle) layout on the host
     const size_t n1 = w1_len(C), n2 = w2_len(C);
-    std::vector<double> gk(n1 + n2), gm(n1 + n2);
-    DWF_CUDA(cudaMemcpyAsync(gk.data(), w.gw, (n1 + n2) * 8, cudaMemcpyDeviceToHost, s));
-    DWF_CUDA(cudaStreamSynchronize(s));
-    for (int d = 0; d < kNDir; ++d)
-        for (int a = 0; a < C; ++a)
-            for (int so = 0; so < 4; ++so)
-                for (int si = 0; si < 4; ++si) {
-                    const size_t m = (((size_t)d * C + a) * 4 + so) * 4 + si;          // master
-                    const size_t k1 = (((size_t)a * 4 + so) * kNDir + d) * 4 + si;      // gW1 kernel
-                    const size_t k2 = (((size_t)d * 4 + so) * C + a) * 4 + si;          // gW2 kernel
-                    gm[2 * m] = gk[2 * k1];
-                    gm[2 * m + 1] = gk[2 * k1 + 1];
-                    gm[n1 + 2 * m] = gk[n1 + 2 * k2];
-                    gm[n1 + 2 * m + 1] = gk[n1 + 2 * k2 + 1];
-                }
-    DWF_CUDA(cudaMemcpyAsync(w.gw, gm.data(), (n1 + n2) * 8, cudaMemcpyHostToDevice, s));
+    for (int p = 0; p < 2; ++p) {
+        const int64_t o = p ? c0 : 0;
+        const int n = kNFold[p];
+        int adj[kNDir];
+        for (int j = 0; j < n; ++j) adj[j] = kAdj[kFoldDirs[p][j]];
+        // g_psi_d = T_d^+ g_z, g_phi_b = sum_d W2[d][b]^+ g_psi_d
+        DWF_TRY(launch_transport(h, nrhs, p, zo, zo, w.psi + o, adj, n, false, s));
+        DWF_TRY(launch_mix(h, nrhs, p, w.psi + o, n, w.gphi + o, C, K->mix2h[p], s));
+        // gW2[d][b] = sum g_psi_d phi_b^+, gW1[a][d] = sum g_phi_a R_d^+
+        if (p == 0) {
+            DWF_TRY((launch_wgrad<kNFold[0], 16>(h, w, nrhs, p, w.psi + o, w.phi + o, true, w.gw + n1, s)));
+            DWF_TRY((launch_wgrad<16, kNFold[0]>(h, w, nrhs, p, w.gphi + o, w.R + o, false, w.gw, s)));
+        } else {
+            DWF_TRY((launch_wgrad<kNFold[1], 16>(h, w, nrhs, p, w.psi + o, w.phi + o, true, w.gw + n1, s)));
+            DWF_TRY((launch_wgrad<16, kNFold[1]>(h, w, nrhs, p, w.gphi + o, w.R + o, false, w.gw, s)));
+        }
+    }
     // Adam (w1 and w2 are separate allocations: two launches over [w1 | w2])
     K->adam_t += 1;
     const float b1 = 0.9f, b2 = 0.999f;
@@ -920,9 +994,8 @@ dwf_status dwf_nn_train_step(dwf_nn* K, dwf_handle* h, const float* r, const flo
                                                     (int)n2, (float)lr, b1, b2, 1e-8f, bc1, bc2);
     note_launch();
     DWF_CUDA(cudaGetLastError());
+    DWF_TRY(refresh_mix(K, s));
     DWF_CUDA(cudaStreamSynchronize(s));
-    cudaFree(d_scal);
-    K->dirty = true;
     return DWF_OK;
 }
 
