@@ -236,6 +236,56 @@ __global__ void k_gather_links(const double* __restrict__ U, const int64_t* __re
     }
 }
 
+// Range of the links' sizes: the biased exponents of the largest element of
+// any link, and of the smallest link's largest element (links of zeros aside);
+// a NaN or infinity has exponent 2047.
+__global__ void k_link_range(const double* __restrict__ l64, int64_t n /* sites * 8 */, int* __restrict__ range) {
+    int hi = 0, lo = 4096;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        int e = 0;
+#pragma unroll
+        for (int j = 0; j < 18; ++j) e = max(e, (__double2hiint(l64[i * 18 + j]) >> 20) & 0x7ff);
+        if (e > 0) {
+            hi = max(hi, e);
+            lo = min(lo, e);
+        }
+    }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&range[0], hi);
+        atomicMin(&range[1], lo);
+    }
+}
+
+// Fixed-point links: w = (hi 2^32 + lo) 2^(exp - 61), lo a signed word, with
+// |w| < 2^exp.  Covered (info[1] = 1): finite links whose sizes differ by at
+// most 2^8, so that the common unit costs none of them precision against FP64
+// (SU(3) links lie within a factor sqrt(3)), of a size that leaves the
+// result's exponent in range.
+__device__ __forceinline__ bool fx_covered(const int* range, int* exp) {
+    *exp = range[0] - 1022;
+    return range[0] > 0 && range[0] - range[1] <= 8 && *exp >= -32 && *exp <= 32;
+}
+
+__global__ void k_fix_links(const double* __restrict__ l64, int64_t n /* reals */, const int* __restrict__ range,
+                            int2* __restrict__ fx) {
+    int exp;
+    if (!fx_covered(range, &exp)) return;
+    const double scale = __hiloint2double((1023 + 61 - exp) << 20, 0);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const long long v = __double2ll_rn(l64[i] * scale);
+        fx[i] = make_int2((int)((v + (1ll << 31)) >> 32), (int)v);
+    }
+}
+
+__global__ void k_fx_info(const int* __restrict__ range, int* __restrict__ info) {
+    int exp;
+    const bool ok = fx_covered(range, &exp);
+    info[0] = ok ? exp : 0;
+    info[1] = ok ? 1 : 0;
+}
+
 // --------------------------------------------------------- layout kernels
 // canonical [box][r][l][s][spin][colour] <-> full field [parity][site][c][r][s]
 template <bool TO_DOMAIN, class S>
@@ -327,7 +377,30 @@ dwf_status set_gauge(dwf_handle* h, const double* U, cudaStream_t s) {
         note_launch();
         DWF_CUDA(cudaGetLastError());
     }
+    // the fixed-point table, where the links' sizes allow it
+    int* range = h->d_fx_info + 2;
+    const int none[2] = {0, 4096};
+    DWF_CUDA(cudaMemcpyAsync(range, none, sizeof(none), cudaMemcpyHostToDevice, s));
+    for (int pass = 0; pass < 2; ++pass)
+        for (int p = 0; p < 2; ++p) {
+            const int64_t n = h->nsite[p] * 8;
+            if (n == 0) continue;
+            const double* l64 = (const double*)h->d_links[0][p];
+            if (pass == 0)
+                k_link_range<<<(int)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(l64, n, range);
+            else
+                k_fix_links<<<(int)std::min<int64_t>((n * 18 + 255) / 256, 152 * 32), 256, 0, s>>>(
+                    l64, n * 18, range, (int2*)h->d_links_fx[p]);
+            note_launch();
+            DWF_CUDA(cudaGetLastError());
+        }
+    k_fx_info<<<1, 1, 0, s>>>(range, h->d_fx_info);
+    note_launch();
+    DWF_CUDA(cudaGetLastError());
+    int info[2] = {0, 0};
+    DWF_CUDA(cudaMemcpyAsync(info, h->d_fx_info, sizeof(info), cudaMemcpyDeviceToHost, s));
     DWF_CUDA(cudaStreamSynchronize(s));
+    h->fx_links = info[1] != 0;
     h->have_gauge = true;
     return DWF_OK;
 }
@@ -513,6 +586,7 @@ dwf_status create(dwf_handle** out, const dwf_params* p, const dwf_box* boxes, i
         if (st == DWF_OK) h->site_local_host[q] = site_local[q];
         for (int pr = 0; pr < 3 && st == DWF_OK; ++pr)
             st = dalloc((char**)&h->d_links[pr][q], ns * 144 * prec_size((dwf_prec)pr));
+        if (st == DWF_OK) st = dalloc(&h->d_links_fx[q], ns * 288);
     }
     if (st == DWF_OK) {
         std::vector<int64_t> bv(2 * h->nbox);
@@ -532,6 +606,7 @@ dwf_status create(dwf_handle** out, const dwf_params* p, const dwf_box* boxes, i
         if (st == DWF_OK)
             st = h2d(h->d_mats, mats.data(), mats.size() * sizeof(float));
     }
+    if (st == DWF_OK) st = dalloc(&h->d_fx_info, 4);
     if (st == DWF_OK) st = dalloc(&h->d_err, 1);
     if (st == DWF_OK) {
         if (cudaMemset(h->d_err, 0, sizeof(int)) != cudaSuccess) {
@@ -646,7 +721,9 @@ dwf_status destroy(dwf_handle* h) {
         cudaFree(h->d_site_box[q]);
         cudaFree(h->d_site_local[q]);
         for (int pr = 0; pr < 3; ++pr) cudaFree(h->d_links[pr][q]);
+        cudaFree(h->d_links_fx[q]);
     }
+    cudaFree(h->d_fx_info);
     cudaFree(h->d_box_canon_vol);
     cudaFree(h->d_err);
     cudaFree(h->d_tmp);

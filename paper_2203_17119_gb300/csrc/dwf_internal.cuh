@@ -31,6 +31,7 @@ using bf16 = __nv_bfloat16;
 constexpr int kMaxLanes = 256;   // Ls * nrhs
 constexpr int kMaxLs = 32;
 constexpr int kHopMaxSmem = 200 * 1024;   // dynamic shared memory cap of the hop
+constexpr int kHopMaxSmemFx = 216 * 1024; // of the fixed-point FP64 hop (more warps' partials)
 constexpr int kMinTile = 4;               // smallest tile the autotuner may pick
 
 // Dynamic shared memory of the register hop: double-buffered links and
@@ -157,6 +158,12 @@ struct dwf_handle {
     int64_t* d_link_src[2] = {nullptr, nullptr}; // [nsite][8] global link or -1
     int64_t* d_box_canon_vol = nullptr;        // [nbox] box volumes
     void* d_links[3][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};
+    // fixed-point form of the FP64 table (hop.cu): [site][8][9] x (re, im) x
+    // (high, low) int32, in units 2^(exponent - 61).  d_fx_info: exponent, 1 if
+    // the loaded links are covered by it, and their size range (set_gauge).
+    int* d_links_fx[2] = {nullptr, nullptr};
+    int* d_fx_info = nullptr;
+    bool fx_links = false;
     bool have_gauge = false;
     std::map<int, dwf::TileSet> tiles;
     int* d_err = nullptr;

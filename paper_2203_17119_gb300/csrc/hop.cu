@@ -32,6 +32,9 @@ struct HopArgs {
     void* out;
     const void* xmoo;
     const void* links;   // parity table [site][8][9] complex (site-major)
+    const double* links64;   // fixed-point hop: the FP64 table, for lanes the fixed point does not cover
+    const int* fx_info;      // fixed-point hop: {link exponent, links covered by the fixed point}
+                             // in device memory, so that a captured launch follows a new gauge field
     const int* nbr;      // [site][8]
     const int4* tiles;
     int T, N5, Ls, nrhs, ntiles;
@@ -364,7 +367,246 @@ __device__ __forceinline__ void hop_dir(const Sin* __restrict__ in, const int* s
     hop_dir_src<K, DAG, Sin, SL, R, VL>(in + ((int64_t)n * 12 * N5 + lane0) * 2, s_link, N5, ar, ai);
 }
 
-// Output of one site's VL lanes: PLAIN out = scale * acc; MOO out = M_oo x +
+// ------------------------------------------------ FP64 hop in fixed point
+// GB300 has 2 FP64 lanes per clock and SM against 32 for the 32 x 32 -> 64-bit
+// integer multiply-add, and the hop's 1320 flops per lane are what bounds the
+// FP64 form (91% of the FP64 pipe).  So the FP64 hop transports in 64-bit
+// fixed point: links as w = (w1 2^32 + w0) 2^(exp - 61), |w1| <= 2^29, w0 a
+// signed word (set_gauge); the projected half spinors h as integers in units
+// of 2^(E - 1080), E one above the largest biased exponent of any component
+// met so far for this site and lane -- so |h| < 2^59 units, and when a larger
+// one arrives the accumulators are shifted to the new unit.  With h = h1 2^32
+// + h0 a real product is three multiply-adds,
+//   w h 2^-64 = w1 h1 + (w1 h0 + w0 h1) 2^-32 + O(2^-2),
+// the second sum enters the first by its high word (rounded: it starts at
+// 2^31), and the colour sum and the sum over directions are integer adds.
+// Bounds: the two product sums stay below 6 2^56 and 6 (2^60 + 2^58) < 2^63,
+// the sum over directions below 2^62, for any |w| <= 1.  A result is within a
+// few of its units, 2^-52 of a component's rms, before one rounding to FP64;
+// FP64 arithmetic rounds every operation by 2^-53, and the error against exact
+// arithmetic comes out no larger than the FP64 form's.  Lanes the fixed point
+// does not cover -- a NaN, an infinity, all components below 2^-895 or one
+// above 2^56 -- run the FP64 form; so does a handle whose links differ in size
+// by more than 2^8 (set_gauge).  Measured, bare hop: 16^4 x 12 650 -> 205 us,
+// 24^4 x 16 4.17 -> 1.34 ms (FP64 form -> this); no pipe is full (FP64 half,
+// integer multiply-add about 60%): the chains of dependent integer
+// instructions at 16 warps per SM are what is left.
+//
+// Half of the projections and conversions (spin 0) run on the FP64 pipe (an
+// add, an exponent add, a conversion), half (spin 1) as shifts of the
+// mantissas: either alone would be the bound.  One body per mu serves both
+// signs, to keep the loop within the instruction cache.
+struct FxLink {
+    int hi, lo;
+};
+
+// |x| of the double v: mantissa aligned to bit 63, moved down by E + 6 - e;
+// EB = (E + 6) << 21 | 0x1fffff
+__device__ __forceinline__ unsigned long long fx_mag(uint2 v, uint32_t EB) {
+    const uint32_t t = (EB - v.y - v.y) >> 21;
+    const uint32_t mh = (v.y & 0xfffffu) | 0x100000u;
+    const unsigned long long m = (((unsigned long long)mh << 32) | v.x) << 11;
+    unsigned long long r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(t));   // 0 beyond 63
+    return r;
+}
+
+// a + b in units of 2^(E - 1080); f = -1: a - b
+__device__ __forceinline__ long long fx_sum(double a, double b, uint32_t EB, int f) {
+    const uint2 va = make_uint2(__double2loint(a), __double2hiint(a)), vb = make_uint2(__double2loint(b), __double2hiint(b));
+    const int sa = (int)va.y >> 31, sb = ((int)vb.y >> 31) ^ f;
+    const unsigned long long ma = fx_mag(va, EB) ^ (unsigned long long)(long long)sa;
+    const unsigned long long mb = fx_mag(vb, EB) ^ (unsigned long long)(long long)sb;
+    return (long long)(ma + mb + (unsigned long long)(uint32_t)(-sa - sb));
+}
+
+// the same on the FP64 pipe, h = a + b given; sh = (1080 - E) << 20, E <= 1080
+// (a zero becomes a number far below one half)
+__device__ __forceinline__ long long fx_conv(double h, int sh) {
+    return __double2ll_rn(__hiloint2double(__double2hiint(h) + sh, __double2loint(h)));
+}
+
+__device__ __forceinline__ long long fx_mad(int a, int b, long long c) { return (long long)a * b + c; }
+
+// acc + g, or acc - g where f = -1
+__device__ __forceinline__ void fx_add(long long& acc, long long g, int f) {
+    acc += (g ^ (long long)f) + (long long)(f & 1);
+}
+
+// Direction +mu (k < 4) or -mu in fixed point: acc += W h on the upper spins,
+// rebuilt lower spins; E the accumulators' unit, bad set where the FP64 form
+// has to decide (denormals only).
+template <int MU, bool DAG>
+__device__ __forceinline__ void hop_dir_fx(int k, const double* __restrict__ in, const int* s_nbr,
+                                           const FxLink* s_link, int N5, int lane0, long long (&ar)[12],
+                                           long long (&ai)[12], int& E, bool& bad) {
+    const int nb = s_nbr[k];
+    if (nb < 0) return;
+    const int P = ((k < 4) != DAG) ? 0 : -1, M = ~P;   // sign masks of +SG and -SG, SG = +1 for (1 - g_mu)
+    const double2* src = reinterpret_cast<const double2*>(in) + ((int64_t)nb * 12 * N5 + lane0);
+    double2 x[12];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) x[c] = __ldg(src + (int64_t)c * N5);
+    // largest magnitude word: the signed maximum sees the positive numbers, the unsigned one the negative
+    int sp = 0;
+    uint32_t sn = 0;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        const int a = __double2hiint(x[c].x), b = __double2hiint(x[c].y);
+        sp = max(sp, max(a, b));
+        sn = max(sn, max((uint32_t)a, (uint32_t)b));
+    }
+    const uint32_t top = max((uint32_t)sp, sn & 0x7fffffffu);
+    const int Ed = (int)(top >> 20);
+    if (top == 0) {   // all zero, or denormals below 2^-1042
+        uint32_t any = 0;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) any |= __double2loint(x[c].x) | __double2loint(x[c].y);
+        if (any) bad = true;
+        return;
+    }
+    if (Ed >= E) {
+        const int d = min(Ed + 1 - E, 63);
+        if (E > 0) {
+#pragma unroll
+            for (int c = 0; c < 12; ++c) { ar[c] >>= d; ai[c] >>= d; }
+        }
+        E = Ed + 1;
+    }
+    const uint32_t EB = ((uint32_t)(E + 6) << 21) | 0x1fffffu;
+    const int sh = (1080 - E) << 20;
+    const double SG = P == 0 ? 1.0 : -1.0;
+    // half spinor h_q = u_q - SG A_mu l: from the other lower spin for mu 0, 1, the same for mu 2, 3; with
+    // a factor i for mu 0, 2; +SG for (mu 1, q 0) and (mu 2, q 1), else -SG; split into signed words
+    constexpr bool ITYPE = MU == 0 || MU == 2;
+    int h1r[2][3], h0r[2][3], h1i[2][3], h0i[2][3];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int low = MU < 2 ? 3 - q : 2 + q;
+        const bool plus = (MU == 1 && q == 0) || (MU == 2 && q == 1);
+        const bool im_plus = ITYPE ? !plus : plus;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double2 u = x[q * 3 + c], l = x[low * 3 + c];
+            const double lr = ITYPE ? l.y : l.x, li = ITYPE ? l.x : l.y;
+            long long r, i;
+            if (q == 0) {
+                r = fx_conv(fma(plus ? SG : -SG, lr, u.x), sh);
+                i = fx_conv(fma(im_plus ? SG : -SG, li, u.y), sh);
+            } else {
+                r = fx_sum(u.x, lr, EB, plus ? P : M);
+                i = fx_sum(u.y, li, EB, im_plus ? P : M);
+            }
+            h0r[q][c] = (int)r;
+            h1r[q][c] = (int)(r >> 32) + (int)((uint32_t)h0r[q][c] >> 31);
+            h0i[q][c] = (int)i;
+            h1i[q][c] = (int)(i >> 32) + (int)((uint32_t)h0i[q][c] >> 31);
+        }
+    }
+    const int4* w = reinterpret_cast<const int4*>(s_link) + k * 9;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int4 v[3] = {w[a * 3], w[a * 3 + 1], w[a * 3 + 2]};   // re high, re low, im high, im low
+        long long qr[2], qi[2], gr[2], gi[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) qr[q] = qi[q] = 0x80000000ll;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int n1 = -v[b].z, n0 = -v[b].w;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                qr[q] = fx_mad(v[b].x, h0r[q][b], qr[q]); qr[q] = fx_mad(v[b].y, h1r[q][b], qr[q]);
+                qr[q] = fx_mad(n1, h0i[q][b], qr[q]); qr[q] = fx_mad(n0, h1i[q][b], qr[q]);
+                qi[q] = fx_mad(v[b].x, h0i[q][b], qi[q]); qi[q] = fx_mad(v[b].y, h1i[q][b], qi[q]);
+                qi[q] = fx_mad(v[b].z, h0r[q][b], qi[q]); qi[q] = fx_mad(v[b].w, h1r[q][b], qi[q]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            gr[q] = (long long)(int)(qr[q] >> 32);
+            gi[q] = (long long)(int)(qi[q] >> 32);
+        }
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int n1 = -v[b].z;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                gr[q] = fx_mad(v[b].x, h1r[q][b], gr[q]); gr[q] = fx_mad(n1, h1i[q][b], gr[q]);
+                gi[q] = fx_mad(v[b].x, h1i[q][b], gi[q]); gi[q] = fx_mad(v[b].z, h1r[q][b], gi[q]);
+            }
+        }
+        // rebuild: upper += g, lower += -SG A_mu^+ g
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int low = MU < 2 ? 3 - q : 2 + q;
+            const bool plus = (MU == 1 && q == 0) || (MU == 2 && q == 1);
+            ar[q * 3 + a] += gr[q];
+            ai[q * 3 + a] += gi[q];
+            if (ITYPE) {
+                fx_add(ar[low * 3 + a], gi[q], plus ? M : P);
+                fx_add(ai[low * 3 + a], gr[q], plus ? P : M);
+            } else {
+                fx_add(ar[low * 3 + a], gr[q], plus ? P : M);
+                fx_add(ai[low * 3 + a], gi[q], plus ? P : M);
+            }
+        }
+    }
+}
+
+// The FP64 form of one site and lane (out of line: rarely taken)
+template <bool DAG>
+__device__ __noinline__ void hop_fx_fallback(const double* in, const int* nb, const double* lk, int N5, int lane0,
+                                             double* r, double* i) {
+    double ar[12][1], ai[12][1];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) ar[c][0] = ai[c][0] = 0.0;
+    hop_dir<0, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai);
+    hop_dir<4, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai);
+    hop_dir<1, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai);
+    hop_dir<5, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai);
+    hop_dir<2, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai);
+    hop_dir<6, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai);
+    hop_dir<3, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai);
+    hop_dir<7, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) { r[c] = ar[c][0]; i[c] = ai[c][0]; }
+}
+
+// Dh of one site and lane: ar, ai times the returned factor
+template <bool DAG>
+__device__ __forceinline__ double hop_site_fx(const double* __restrict__ in, const int* nb, const FxLink* lk,
+                                              const double* lk64, int2 info, int N5, int lane0,
+                                              double (&ar)[12][1], double (&ai)[12][1]) {
+    long long r[12], i[12];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) r[c] = i[c] = 0;
+    int E = 0;
+    bool bad = false;
+#pragma unroll 1
+    for (int k = 0; k < 8; k += 4) hop_dir_fx<0, DAG>(k, in, nb, lk, N5, lane0, r, i, E, bad);
+#pragma unroll 1
+    for (int k = 1; k < 8; k += 4) hop_dir_fx<1, DAG>(k, in, nb, lk, N5, lane0, r, i, E, bad);
+#pragma unroll 1
+    for (int k = 2; k < 8; k += 4) hop_dir_fx<2, DAG>(k, in, nb, lk, N5, lane0, r, i, E, bad);
+#pragma unroll 1
+    for (int k = 3; k < 8; k += 4) hop_dir_fx<3, DAG>(k, in, nb, lk, N5, lane0, r, i, E, bad);
+    // E = 0: every neighbour component is zero (or the FP64 form runs)
+    if (((E != 0 || bad) && (E < 128 || E > 1080)) || info.y == 0) {
+        double tr[12], ti[12];
+        hop_fx_fallback<DAG>(in, nb, lk64, N5, lane0, tr, ti);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) { ar[c][0] = tr[c]; ai[c][0] = ti[c]; }
+        return 1.0;
+    }
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        ar[c][0] = __ll2double_rn(r[c]);
+        ai[c][0] = __ll2double_rn(i[c]);
+    }
+    return __hiloint2double(max(E + info.x - 54, 1) << 20, 0);   // 2^(E + exp - 1077)
+}
+
+// Output of one site's VL lanes (acc = factor (ar, ai)): PLAIN out = scale * acc; MOO out = M_oo x +
 // scale * acc, returning the lanes' |out|^2 (FP32 arithmetic: summed in FP32
 // per site, one FP64 add per site, off GB300's slow FP64 pipe).
 // Site groups (N5 / VL threads) known at compile time to divide a warp: the
@@ -374,9 +616,9 @@ constexpr bool kLaneShfl = CN5 > 0 && CN5 % VL == 0 && CN5 / VL <= 32 && 32 % (C
 
 template <class Sout, class R, int VL, bool DAG, int EPI, int CN5>
 __device__ __forceinline__ double hop_store(const HopArgs& a, int N5, int64_t site, int lane0,
-                                            const R (&ar)[12][VL], const R (&ai)[12][VL],
+                                            const R (&ar)[12][VL], const R (&ai)[12][VL], R factor,
                                             const LaneNbrs& nb, int box, const ScanCtx<VL>& sk) {
-    const R sc = (R)a.scale;
+    const R sc = (R)a.scale * factor;
     if constexpr (EPI == EPI_BMINV) {
         // out = scale B M^-1 acc: non-adjoint upper spins see S_-, lower S_+
         Sout* out = reinterpret_cast<Sout*>(a.out) + (site * 12 * N5 + lane0) * 2;
@@ -535,7 +777,8 @@ __device__ __forceinline__ double hop_store(const HopArgs& a, int N5, int64_t si
             // the neighbouring lane is held by the adjacent thread of the site group
             nr = __shfl_sync(nb.mask, use_below ? xr[VL - 1] : xr[0], use_below ? nb.src_dn : nb.src_up);
             ni = __shfl_sync(nb.mask, use_below ? xi[VL - 1] : xi[0], use_below ? nb.src_dn : nb.src_up);
-            fn = (R)(use_below ? nb.f_dn : nb.f_up);
+            if constexpr (sizeof(R) == 8) fn = use_below ? f_below : f_above;   // (nb's factors are FP32)
+            else fn = (R)(use_below ? nb.f_dn : nb.f_up);
         } else {
             load_c1<Sout, R>(xb + (int64_t)(c * N5 + (use_below ? l_below : l_above)) * 2, nr, ni);
             fn = use_below ? f_below : f_above;
@@ -555,7 +798,7 @@ __device__ __forceinline__ double hop_store(const HopArgs& a, int N5, int64_t si
             orr[v] = d * xr[v] + e * sr + sc * ar[c][v];
             oi[v] = d * xi[v] + e * si + sc * ai[c][v];
             part += (float)(orr[v] * orr[v] + oi[v] * oi[v]);
-            if (sizeof(R) == 8) nrm += (double)orr[v] * orr[v] + (double)oi[v] * oi[v];
+            if (sizeof(R) == 8 && a.partial != nullptr) nrm += (double)orr[v] * orr[v] + (double)oi[v] * oi[v];
         }
         if (sizeof(R) != 8) nrm_f += part;
         store_lanes<Sout, VL, R, true>(out + (int64_t)c * N5 * 2, orr, oi);
@@ -572,8 +815,18 @@ __device__ __forceinline__ double hop_store(const HopArgs& a, int N5, int64_t si
 // fast warps run on into the next tile.
 // CN5 > 0 fixes N5 = Ls * nrhs at compile time (the common single-rhs
 // cases), so the row offsets of every spinor load and store are immediates.
+// Threads per CTA: 256, two or three CTAs per SM; the fixed-point FP64 hop, one
+// CTA of 512 (128 registers and some 30 bytes of spills: 1.34 ms at 24^4 x 16,
+// against 1.53 with 384 threads of 168 registers and 1.67 with 2 x 192).
+template <class SL>
+constexpr int kHopThreads = std::is_same<SL, FxLink>::value ? 512 : 256;
+
 template <class Sin, class Sout, class SL, class R, int VL, bool DAG, int EPI, int CN5>
-__global__ void __launch_bounds__(256, (VL == 1 && sizeof(R) == 4) ? 3 : 2) k_hop(const HopArgs a) {
+__global__ void __launch_bounds__(kHopThreads<SL>, std::is_same<SL, FxLink>::value       ? 1
+                                                   : (VL == 1 && sizeof(R) == 4) ? 3
+                                                                                         : 2)
+k_hop(const HopArgs a) {
+    constexpr bool FX = std::is_same<SL, FxLink>::value;
     extern __shared__ __align__(128) unsigned char smem[];
     const int N5 = CN5 > 0 ? CN5 : a.N5;
     const int TPS = N5 / VL;
@@ -665,6 +918,9 @@ __global__ void __launch_bounds__(256, (VL == 1 && sizeof(R) == 4) ? 3 : 2) k_ho
     }
 
     int k = 0;
+    const int2 fx_info = FX ? *reinterpret_cast<const int2*>(a.fx_info) : make_int2(0, 0);
+    int turn = 0;   // fixed-point hop: sites done so far mod G, so that the groups that
+                    // take a tile's remainder change from tile to tile
     for (int tile = tile_of(0); tile < nt; tile = tile_of(++k)) {
         const int b = k & 1;
         const uint32_t ph = (uint32_t)((k >> 1) & 1);
@@ -681,7 +937,12 @@ __global__ void __launch_bounds__(256, (VL == 1 && sizeof(R) == 4) ? 3 : 2) k_ho
         const SL* s_link_t = reinterpret_cast<const SL*>(smem + b * buf_bytes);
         const int* s_nbr_t = reinterpret_cast<const int*>(smem + b * buf_bytes + link_bytes);
         double tile_norm = 0.0;
-        for (int sl = sg; sg < G && sl < count; sl += G) {
+        int first = sg;
+        if constexpr (FX) {
+            first = sg - turn + (sg < turn ? G : 0);
+            turn = (turn + count) % G;
+        }
+        for (int sl = first; sg < G && sl < count; sl += G) {
             // the M_oo input of this site's lanes, into L1 while the last two
             // directions run (earlier, the lines are evicted by the neighbour
             // traffic before the epilogue reads them)
@@ -694,12 +955,16 @@ __global__ void __launch_bounds__(256, (VL == 1 && sizeof(R) == 4) ? 3 : 2) k_ho
                 }
             };
             R ar[12][VL], ai[12][VL];
+            R factor = (R)1;
             const Sin* in = reinterpret_cast<const Sin*>(a.in);
             const int* nb = s_nbr_t + sl * 8;
             const SL* lk = s_link_t + (size_t)sl * 144;
             // +mu and -mu back to back: the row that is the +x neighbour of
             // one site is the -x neighbour of the next, still in L1
-            if constexpr (std::is_same<R, float>::value && VL == 2 && std::is_same<Sin, bf16>::value) {
+            if constexpr (FX) {
+                factor = hop_site_fx<DAG>(in, nb, lk, a.links64 + (int64_t)(begin + sl) * 144, fx_info, N5, lane0, ar,
+                                          ai);
+            } else if constexpr (std::is_same<R, float>::value && VL == 2 && std::is_same<Sin, bf16>::value) {
                 float2 pr[12], pi[12];
 #pragma unroll
                 for (int c = 0; c < 12; ++c) pr[c] = pi[c] = make_float2(0.f, 0.f);
@@ -732,7 +997,7 @@ __global__ void __launch_bounds__(256, (VL == 1 && sizeof(R) == 4) ? 3 : 2) k_ho
                 hop_dir<3, DAG, Sin, SL, R, VL>(in, nb, lk, N5, lane0, ar, ai);
                 hop_dir<7, DAG, Sin, SL, R, VL>(in, nb, lk, N5, lane0, ar, ai);
             }
-            tile_norm += hop_store<Sout, R, VL, DAG, EPI, CN5>(a, N5, begin + sl, lane0, ar, ai, nbrs, tl.x, sk);
+            tile_norm += hop_store<Sout, R, VL, DAG, EPI, CN5>(a, N5, begin + sl, lane0, ar, ai, factor, nbrs, tl.x, sk);
         }
         double* red = s_red + (size_t)b * nwarps * a.nrhs;
         if (part) {
@@ -770,7 +1035,10 @@ static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, c
     a.in = c.in;
     a.out = c.out;
     a.xmoo = c.xmoo;
-    a.links = h->d_links[c.prec_link][p];
+    constexpr bool FX = std::is_same<SL, FxLink>::value;
+    a.links = FX ? h->d_links_fx[p] : h->d_links[c.prec_link][p];
+    a.links64 = static_cast<const double*>(h->d_links[DWF_FP64][p]);
+    a.fx_info = h->d_fx_info;
     a.nbr = h->d_nbr[p];
     a.tiles = ts.d_tiles[p];
     a.T = ts.T;
@@ -795,11 +1063,13 @@ static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, c
     a.alpha = c.alpha;
     a.run = c.run;
     const int TPS = a.N5 / VL;
-    // site groups per CTA: as many as fit in 256 threads, at most T
-    int groups = 256 / TPS;
-    if (groups > ts.T) groups = ts.T;
+    // site groups per CTA: as many as fit in its threads, at most T (the
+    // fixed-point hop deals sites out in turn across tiles: as many as the two
+    // buffered tiles hold)
+    int groups = kHopThreads<SL> / TPS;
+    if (groups > (FX ? 2 : 1) * ts.T) groups = (FX ? 2 : 1) * ts.T;
     if (groups < 1) {
-        set_error("hop: %d threads per site exceed 256", TPS);
+        set_error("hop: %d threads per site exceed %d", TPS, kHopThreads<SL>);
         return DWF_ERR_ARG;
     }
     int threads = (groups * TPS + 31) / 32 * 32;
@@ -840,7 +1110,7 @@ static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, c
     else
         kern = moo ? k_hop<Sin, Sout, SL, R, VL, false, EPI_MOO, CN5>
                    : k_hop<Sin, Sout, SL, R, VL, false, EPI_PLAIN, CN5>;
-    if (smem > kHopMaxSmem) {
+    if (smem > (FX ? kHopMaxSmemFx : kHopMaxSmem)) {
         set_error("hop: tile of %d sites needs %zu bytes of shared memory", ts.T, smem);
         return DWF_ERR_ARG;
     }
@@ -885,7 +1155,8 @@ static cudaError_t hop_attr() {
                                    k_hop<Sin, Sout, SL, R, VL, true, EPI_PLAIN, CN5>,
                                    k_hop<Sin, Sout, SL, R, VL, true, EPI_MOO, CN5>};
     for (auto f : k) {
-        cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kHopMaxSmem);
+        cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             std::is_same<SL, FxLink>::value ? kHopMaxSmemFx : kHopMaxSmem);
         if (r != cudaSuccess) e = r;
     }
     if constexpr (std::is_same<R, float>::value && std::is_same<Sout, float>::value) {
@@ -906,6 +1177,9 @@ static cudaError_t hop_attr() {
 
 dwf_status init_hop_kernels() {
     DWF_CUDA((hop_attr<double, double, double, double, 1>()));
+    DWF_CUDA((hop_attr<double, double, FxLink, double, 1>()));
+    DWF_CUDA((hop_attr<double, double, FxLink, double, 1, 12>()));
+    DWF_CUDA((hop_attr<double, double, FxLink, double, 1, 16>()));
     DWF_CUDA((hop_attr<float, float, float, float, 2>()));
     DWF_CUDA((hop_attr<float, float, float, float, 1>()));
     DWF_CUDA((hop_attr<bf16, bf16, bf16, float, 2>()));
@@ -943,6 +1217,12 @@ dwf_status launch_hop(dwf_handle* h, const HopCall& c, cudaStream_t s) {
     const TileSet& ts = *tsp;
     if (c.prec_link == DWF_FP64) {
         if (c.prec_in != DWF_FP64 || c.prec_out != DWF_FP64) return DWF_ERR_UNSUPPORTED;
+        if (h->fx_links) {
+            const int N5 = h->p.Ls * c.nrhs;
+            if (N5 == 12) return launch_t<double, double, FxLink, double, 1, 12>(h, c, ts, s);
+            if (N5 == 16) return launch_t<double, double, FxLink, double, 1, 16>(h, c, ts, s);
+            return launch_t<double, double, FxLink, double, 1>(h, c, ts, s);
+        }
         return launch_t<double, double, double, double, 1>(h, c, ts, s);
     }
     if (c.prec_link == DWF_FP32) {
