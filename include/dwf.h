@@ -275,7 +275,8 @@ dwf_status dwf_cgne_solve(dwf_handle* h, double* x, const double* b, int nrhs,
                           void* stream);
 
 /* Autotuner: time the hop kernel for nrhs right-hand sides in precision
- * `prec` over candidate tile sizes (sites per CTA tile: 8..128) and keep the
+ * `prec` over candidate tile sizes (sites per CTA tile: 8..128, 4 on small
+ * domains) and keep the
  * fastest for every later call on this handle with that nrhs (all kernels of
  * an operator chain share one tile table).  On a whole-lattice handle it then
  * times the chosen configuration with the lexicographic and the 8 x 8 blocked
@@ -349,7 +350,8 @@ dwf_status dwf_set_tile_order(dwf_handle* h, int order, int bz, int bt);
 dwf_status dwf_get_tile_order(const dwf_handle* h, int* order, int* bz, int* bt);
 
 /* The kernel configuration later calls with this nrhs use (set by
- * dwf_autotune or the dwf_set_* calls; defaults 32 sites, 2 lanes, chunk 1,
+ * dwf_autotune or the dwf_set_* calls; defaults 32 sites -- fewer, down to 4,
+ * on a domain of fewer than 304 such tiles a parity --, 2 lanes, chunk 1,
  * SIMT): any output pointer may be NULL.  DWF_ERR_ARG on a bad nrhs. */
 dwf_status dwf_get_tuning(const dwf_handle* h, int nrhs, int* tile_sites, int* lanes_per_thread,
                           int* chunk, int* tensor_cores);

@@ -341,7 +341,7 @@ dwf_status dwf_get_tuning(const dwf_handle* h, int nrhs, int* tile_sites, int* l
         auto it = m.find(nrhs);
         return it == m.end() ? dflt : it->second;
     };
-    if (tile_sites) *tile_sites = get(h->tuned_T, 32);
+    if (tile_sites) *tile_sites = get(h->tuned_T, h->default_T);
     if (lanes_per_thread) *lanes_per_thread = get(h->tuned_vl, 2);
     if (chunk) *chunk = get(h->tuned_chunk, 1);
     if (tensor_cores) *tensor_cores = get(h->tuned_tc, 0);

@@ -618,8 +618,14 @@ dwf_status create(dwf_handle** out, const dwf_params* p, const dwf_box* boxes, i
         if (st == DWF_OK) st = dalloc((double**)&h->d_tmp2, nmax);
     }
     if (st == DWF_OK) {   // default tile table, built up front
+        // 32 sites, halved (to 4 at least) while a parity has fewer tiles than two
+        // per SM: an SM works on one tile at a time, and a tile's rows are a chain
+        // of passes for its CTA (FP64 CGNE on 4^4 x 8: 4 tiles of 32 kept 4 of 152
+        // SMs busy)
+        const int64_t ns = std::max(h->nsite[0], h->nsite[1]);
+        while (h->default_T > kMinTile && (ns + h->default_T - 1) / h->default_T < 2 * 152) h->default_T /= 2;
         const TileSet* ts = nullptr;
-        st = get_tiles(h, 32, &ts);
+        st = get_tiles(h, h->default_T, &ts);
     }
     if (st == DWF_OK) {
         cudaError_t e = cudaDeviceSynchronize();

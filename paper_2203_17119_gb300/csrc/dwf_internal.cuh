@@ -166,6 +166,7 @@ struct dwf_handle {
     bool fx_links = false;
     bool have_gauge = false;
     std::map<int, dwf::TileSet> tiles;
+    int default_T = 32;           // sites per tile until dwf_autotune or dwf_set_tile chooses
     int* d_err = nullptr;
     void* d_tmp = nullptr;        // one FP64 cb field x nrhs_max (operator calls)
     void* d_tmp2 = nullptr;
@@ -337,6 +338,7 @@ struct LocalCall {
     const FiveD* f5 = nullptr;   // FP64 only: fifth-dimension coefficients other than the handle's
 };
 dwf_status launch_local(dwf_handle* h, const LocalCall& c, cudaStream_t s);
+dwf_status launch_local64(dwf_handle* h, const LocalCall& c, const TileSet& ts, cudaStream_t s);   // FP64
 
 // elementwise / reduction kernels (blas.cu)
 // copy between device and page-locked host memory with SM loads and stores

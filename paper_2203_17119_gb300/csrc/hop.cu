@@ -26,7 +26,6 @@
 #include "dwf_internal.cuh"
 
 namespace dwf {
-
 struct HopArgs {
     const void* in;
     void* out;
@@ -433,21 +432,22 @@ __device__ __forceinline__ void fx_add(long long& acc, long long g, int f) {
     acc += (g ^ (long long)f) + (long long)(f & 1);
 }
 
-// Direction +mu (k < 4) or -mu in fixed point: acc += W h on the upper spins,
-// rebuilt lower spins; E the accumulators' unit, bad set where the FP64 form
-// has to decide (denormals only).
-template <int MU, bool DAG>
-__device__ __forceinline__ void hop_dir_fx(int k, const double* __restrict__ in, const int* s_nbr,
-                                           const FxLink* s_link, int N5, int lane0, long long (&ar)[12],
-                                           long long (&ai)[12], int& E, bool& bad) {
-    const int nb = s_nbr[k];
-    if (nb < 0) return;
-    const int P = ((k < 4) != DAG) ? 0 : -1, M = ~P;   // sign masks of +SG and -SG, SG = +1 for (1 - g_mu)
-    const double2* src = reinterpret_cast<const double2*>(in) + ((int64_t)nb * 12 * N5 + lane0);
-    double2 x[12];
-#pragma unroll
-    for (int c = 0; c < 12; ++c) x[c] = __ldg(src + (int64_t)c * N5);
-    // largest magnitude word: the signed maximum sees the positive numbers, the unsigned one the negative
+// Spin structure of one direction: the half spinor h_q = u_q - SG A_mu l takes
+// lower spin fx_low(MU, q), with a factor i for mu 0, 2, and sign +SG for
+// (mu 1, q 0) and (mu 2, q 1), else -SG; -SG A_mu^+ g puts g_q back there.
+__host__ __device__ constexpr int fx_low(int mu, int q) { return mu < 2 ? 3 - q : 2 + q; }
+__host__ __device__ constexpr bool fx_itype(int mu) { return mu == 0 || mu == 2; }
+__host__ __device__ constexpr bool fx_plus(int mu, int q) { return (mu == 1 && q == 0) || (mu == 2 && q == 1); }
+
+// a half spinor split into signed words
+struct FxHalf {
+    int h1r[2][3], h0r[2][3], h1i[2][3], h0i[2][3];
+};
+
+// largest magnitude word of a neighbour's components, 0 if all are zero (or
+// denormals below 2^-1042, which set bad): the signed maximum sees the
+// positive numbers, the unsigned one the negative
+__device__ __forceinline__ uint32_t fx_top(const double2 (&x)[12], bool& bad) {
     int sp = 0;
     uint32_t sn = 0;
 #pragma unroll
@@ -457,38 +457,30 @@ __device__ __forceinline__ void hop_dir_fx(int k, const double* __restrict__ in,
         sn = max(sn, max((uint32_t)a, (uint32_t)b));
     }
     const uint32_t top = max((uint32_t)sp, sn & 0x7fffffffu);
-    const int Ed = (int)(top >> 20);
-    if (top == 0) {   // all zero, or denormals below 2^-1042
+    if (top == 0) {
         uint32_t any = 0;
 #pragma unroll
         for (int c = 0; c < 12; ++c) any |= __double2loint(x[c].x) | __double2loint(x[c].y);
         if (any) bad = true;
-        return;
     }
-    if (Ed >= E) {
-        const int d = min(Ed + 1 - E, 63);
-        if (E > 0) {
-#pragma unroll
-            for (int c = 0; c < 12; ++c) { ar[c] >>= d; ai[c] >>= d; }
-        }
-        E = Ed + 1;
-    }
+    return top;
+}
+
+// The half spinor of direction MU in the unit of E; P, M = ~P the sign masks
+// of +SG and -SG.
+template <int MU>
+__device__ __forceinline__ void fx_project(const double2 (&x)[12], int P, int E, FxHalf& h) {
+    const int M = ~P;
     const uint32_t EB = ((uint32_t)(E + 6) << 21) | 0x1fffffu;
     const int sh = (1080 - E) << 20;
     const double SG = P == 0 ? 1.0 : -1.0;
-    // half spinor h_q = u_q - SG A_mu l: from the other lower spin for mu 0, 1, the same for mu 2, 3; with
-    // a factor i for mu 0, 2; +SG for (mu 1, q 0) and (mu 2, q 1), else -SG; split into signed words
-    constexpr bool ITYPE = MU == 0 || MU == 2;
-    int h1r[2][3], h0r[2][3], h1i[2][3], h0i[2][3];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-        const int low = MU < 2 ? 3 - q : 2 + q;
-        const bool plus = (MU == 1 && q == 0) || (MU == 2 && q == 1);
-        const bool im_plus = ITYPE ? !plus : plus;
+        const bool plus = fx_plus(MU, q), im_plus = fx_itype(MU) ? !plus : plus;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double2 u = x[q * 3 + c], l = x[low * 3 + c];
-            const double lr = ITYPE ? l.y : l.x, li = ITYPE ? l.x : l.y;
+            const double2 u = x[q * 3 + c], l = x[fx_low(MU, q) * 3 + c];
+            const double lr = fx_itype(MU) ? l.y : l.x, li = fx_itype(MU) ? l.x : l.y;
             long long r, i;
             if (q == 0) {
                 r = fx_conv(fma(plus ? SG : -SG, lr, u.x), sh);
@@ -497,57 +489,92 @@ __device__ __forceinline__ void hop_dir_fx(int k, const double* __restrict__ in,
                 r = fx_sum(u.x, lr, EB, plus ? P : M);
                 i = fx_sum(u.y, li, EB, im_plus ? P : M);
             }
-            h0r[q][c] = (int)r;
-            h1r[q][c] = (int)(r >> 32) + (int)((uint32_t)h0r[q][c] >> 31);
-            h0i[q][c] = (int)i;
-            h1i[q][c] = (int)(i >> 32) + (int)((uint32_t)h0i[q][c] >> 31);
+            h.h0r[q][c] = (int)r;
+            h.h1r[q][c] = (int)(r >> 32) + (int)((uint32_t)h.h0r[q][c] >> 31);
+            h.h0i[q][c] = (int)i;
+            h.h1i[q][c] = (int)(i >> 32) + (int)((uint32_t)h.h0i[q][c] >> 31);
         }
     }
+}
+
+// Row v (re high, re low, im high, im low of three links) times the two half spinors
+__device__ __forceinline__ void fx_row(const int4 (&v)[3], const FxHalf& h, long long (&gr)[2], long long (&gi)[2]) {
+    long long qr[2], qi[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) qr[q] = qi[q] = 0x80000000ll;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const int n1 = -v[b].z, n0 = -v[b].w;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            qr[q] = fx_mad(v[b].x, h.h0r[q][b], qr[q]); qr[q] = fx_mad(v[b].y, h.h1r[q][b], qr[q]);
+            qr[q] = fx_mad(n1, h.h0i[q][b], qr[q]); qr[q] = fx_mad(n0, h.h1i[q][b], qr[q]);
+            qi[q] = fx_mad(v[b].x, h.h0i[q][b], qi[q]); qi[q] = fx_mad(v[b].y, h.h1i[q][b], qi[q]);
+            qi[q] = fx_mad(v[b].z, h.h0r[q][b], qi[q]); qi[q] = fx_mad(v[b].w, h.h1r[q][b], qi[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        gr[q] = (long long)(int)(qr[q] >> 32);
+        gi[q] = (long long)(int)(qi[q] >> 32);
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const int n1 = -v[b].z;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            gr[q] = fx_mad(v[b].x, h.h1r[q][b], gr[q]); gr[q] = fx_mad(n1, h.h1i[q][b], gr[q]);
+            gi[q] = fx_mad(v[b].x, h.h1i[q][b], gi[q]); gi[q] = fx_mad(v[b].z, h.h1r[q][b], gi[q]);
+        }
+    }
+}
+
+// Direction +mu (k < 4) or -mu in fixed point: acc += W h on the upper spins,
+// rebuilt lower spins; E the accumulators' unit, bad set where the FP64 form
+// has to decide (denormals only).
+template <int MU, bool DAG>
+__device__ __forceinline__ void hop_dir_fx(int k, const double* __restrict__ in, const int* s_nbr,
+                                           const FxLink* s_link, int N5, int lane0, long long (&ar)[12],
+                                           long long (&ai)[12], int& E, bool& bad) {
+    const int nb = s_nbr[k];
+    if (nb < 0) return;
+    const int P = ((k < 4) != DAG) ? 0 : -1, M = ~P;   // SG = +1 for (1 - g_mu)
+    const double2* src = reinterpret_cast<const double2*>(in) + ((int64_t)nb * 12 * N5 + lane0);
+    double2 x[12];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) x[c] = __ldg(src + (int64_t)c * N5);
+    const uint32_t top = fx_top(x, bad);
+    if (top == 0) return;
+    const int Ed = (int)(top >> 20);
+    if (Ed >= E) {
+        const int d = min(Ed + 1 - E, 63);
+        if (E > 0) {
+#pragma unroll
+            for (int c = 0; c < 12; ++c) { ar[c] >>= d; ai[c] >>= d; }
+        }
+        E = Ed + 1;
+    }
+    FxHalf h;
+    fx_project<MU>(x, P, E, h);
     const int4* w = reinterpret_cast<const int4*>(s_link) + k * 9;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const int4 v[3] = {w[a * 3], w[a * 3 + 1], w[a * 3 + 2]};   // re high, re low, im high, im low
-        long long qr[2], qi[2], gr[2], gi[2];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) qr[q] = qi[q] = 0x80000000ll;
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const int n1 = -v[b].z, n0 = -v[b].w;
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                qr[q] = fx_mad(v[b].x, h0r[q][b], qr[q]); qr[q] = fx_mad(v[b].y, h1r[q][b], qr[q]);
-                qr[q] = fx_mad(n1, h0i[q][b], qr[q]); qr[q] = fx_mad(n0, h1i[q][b], qr[q]);
-                qi[q] = fx_mad(v[b].x, h0i[q][b], qi[q]); qi[q] = fx_mad(v[b].y, h1i[q][b], qi[q]);
-                qi[q] = fx_mad(v[b].z, h0r[q][b], qi[q]); qi[q] = fx_mad(v[b].w, h1r[q][b], qi[q]);
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            gr[q] = (long long)(int)(qr[q] >> 32);
-            gi[q] = (long long)(int)(qi[q] >> 32);
-        }
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const int n1 = -v[b].z;
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                gr[q] = fx_mad(v[b].x, h1r[q][b], gr[q]); gr[q] = fx_mad(n1, h1i[q][b], gr[q]);
-                gi[q] = fx_mad(v[b].x, h1i[q][b], gi[q]); gi[q] = fx_mad(v[b].z, h1r[q][b], gi[q]);
-            }
-        }
+        const int4 v[3] = {w[a * 3], w[a * 3 + 1], w[a * 3 + 2]};
+        long long gr[2], gi[2];
+        fx_row(v, h, gr, gi);
         // rebuild: upper += g, lower += -SG A_mu^+ g
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            const int low = MU < 2 ? 3 - q : 2 + q;
-            const bool plus = (MU == 1 && q == 0) || (MU == 2 && q == 1);
+            const int low = fx_low(MU, q) * 3 + a;
+            const bool plus = fx_plus(MU, q);
             ar[q * 3 + a] += gr[q];
             ai[q * 3 + a] += gi[q];
-            if (ITYPE) {
-                fx_add(ar[low * 3 + a], gi[q], plus ? M : P);
-                fx_add(ai[low * 3 + a], gr[q], plus ? P : M);
+            if (fx_itype(MU)) {
+                fx_add(ar[low], gi[q], plus ? M : P);
+                fx_add(ai[low], gr[q], plus ? P : M);
             } else {
-                fx_add(ar[low * 3 + a], gr[q], plus ? P : M);
-                fx_add(ai[low * 3 + a], gi[q], plus ? P : M);
+                fx_add(ar[low], gr[q], plus ? P : M);
+                fx_add(ai[low], gi[q], plus ? P : M);
             }
         }
     }
@@ -1027,15 +1054,161 @@ k_hop(const HopArgs a) {
     }
 }
 
+// The fixed-point FP64 hop on a domain too small to fill the chip: there a
+// lane's chain of eight directions, ~20 us, is the whole time.  Warp k of a CTA takes direction k of 32 lanes of its tile,
+// and warps 0..5 add the eight directions' half spinors from shared memory,
+// two spin-colour rows each, in the largest of the eight units.
+// 4^4 x 8 (1024 lanes): 20.5 us -> 7.9 with the call's launch.
+constexpr int kSplitLanes = 32;
+
+template <bool DAG, int EPI>
+__global__ void __launch_bounds__(256, 2) k_hop_fx_split(const HopArgs a) {
+    __shared__ long long s_g[8][12][kSplitLanes];   // [direction][(q * 3 + colour) * 2 + part][lane]
+    __shared__ int s_E[8][kSplitLanes];             // unit, 0: nothing, -1: the FP64 form decides
+    __shared__ double s_red[256];
+    __shared__ double s_sum[kMaxLanes / 2];
+    const int N5 = a.N5, Ls = a.Ls, nrhs = a.nrhs;
+    const int4 tl = a.tiles[blockIdx.x];
+    const int items = tl.z * N5;
+    const int k = threadIdx.x >> 5, j = threadIdx.x & 31;
+    const int2 info = *reinterpret_cast<const int2*>(a.fx_info);
+    const double* in = reinterpret_cast<const double*>(a.in);
+    const bool part = EPI == EPI_MOO && a.partial != nullptr;
+    if (part)
+        for (int r = threadIdx.x; r < nrhs; r += blockDim.x) s_sum[r] = 0.0;
+    for (int g0 = 0; g0 < items; g0 += kSplitLanes) {
+        const bool on = g0 + j < items;
+        const int item = on ? g0 + j : 0;
+        const int64_t site = tl.y + item / N5;
+        const int lane0 = item % N5;
+        const int nb = on ? a.nbr[site * 8 + k] : -1;
+        int E = 0;
+        if (nb >= 0) {
+            const double2* src = reinterpret_cast<const double2*>(in) + ((int64_t)nb * 12 * N5 + lane0);
+            double2 x[12];
+#pragma unroll
+            for (int c = 0; c < 12; ++c) x[c] = __ldg(src + (int64_t)c * N5);
+            bool bad = false;
+            const uint32_t top = fx_top(x, bad);
+            if (bad) E = -1;
+            if (top != 0) {
+                E = (int)(top >> 20) + 1;
+                const int P = ((k < 4) != DAG) ? 0 : -1;
+                FxHalf h;
+                switch (k & 3) {   // the same for the whole warp
+                    case 0: fx_project<0>(x, P, E, h); break;
+                    case 1: fx_project<1>(x, P, E, h); break;
+                    case 2: fx_project<2>(x, P, E, h); break;
+                    default: fx_project<3>(x, P, E, h);
+                }
+                const int4* w = reinterpret_cast<const int4*>(a.links) + (site * 8 + k) * 9;
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    const int4 v[3] = {__ldg(w + r * 3), __ldg(w + r * 3 + 1), __ldg(w + r * 3 + 2)};
+                    long long gr[2], gi[2];
+                    fx_row(v, h, gr, gi);
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        s_g[k][(q * 3 + r) * 2][j] = gr[q];
+                        s_g[k][(q * 3 + r) * 2 + 1][j] = gi[q];
+                    }
+                }
+            }
+        }
+        s_E[k][j] = E;
+        __syncthreads();
+        double nrm = 0.0;
+        if (k < 6 && on) {
+            int Em = 0;
+            bool bad = false;
+#pragma unroll
+            for (int d = 0; d < 8; ++d) {
+                Em = max(Em, s_E[d][j]);
+                bad |= s_E[d][j] < 0;
+            }
+            double re[2], im[2], factor;
+            if (((Em != 0 || bad) && (Em < 128 || Em > 1080)) || info.y == 0) {
+                double tr[12], ti[12];
+                hop_fx_fallback<DAG>(in, a.nbr + site * 8, a.links64 + site * 144, N5, lane0, tr, ti);
+#pragma unroll
+                for (int c = 0; c < 12; ++c)
+                    if (c >> 1 == k) { re[c & 1] = tr[c]; im[c & 1] = ti[c]; }
+                factor = 1.0;
+            } else {
+                const bool upper = k < 3;   // rows 2 k, 2 k + 1: upper spins for k < 3
+                long long sr[2] = {0, 0}, si[2] = {0, 0};
+#pragma unroll
+                for (int d = 0; d < 8; ++d) {
+                    const int Ek = s_E[d][j];
+                    if (Ek <= 0) continue;
+                    const int dn = min(Em - Ek, 63);
+                    const int P = ((d < 4) != DAG) ? 0 : -1, mu = d & 3;
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int c = 2 * k + e, spin = c / 3, col = c - 3 * spin;
+                        const int q = upper ? spin : (mu < 2 ? 3 - spin : spin - 2);
+                        const long long gr = s_g[d][(q * 3 + col) * 2][j] >> dn, gi = s_g[d][(q * 3 + col) * 2 + 1][j] >> dn;
+                        if (upper) {
+                            sr[e] += gr;
+                            si[e] += gi;
+                        } else {
+                            const int f = fx_plus(mu, q) ? P : ~P;   // sign mask of the term (of its im part for i types)
+                            if (fx_itype(mu)) { fx_add(sr[e], gi, ~f); fx_add(si[e], gr, f); }
+                            else { fx_add(sr[e], gr, f); fx_add(si[e], gi, f); }
+                        }
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < 2; ++e) { re[e] = __ll2double_rn(sr[e]); im[e] = __ll2double_rn(si[e]); }
+                factor = __hiloint2double(max(Em + info.x - 54, 1) << 20, 0);
+            }
+            const double sc = a.scale * factor;
+            const int s = lane0 % Ls;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int c = 2 * k + e;
+                const int64_t row = (site * 12 + c) * N5;
+                double yr = sc * re[e], yi = sc * im[e];
+                if (EPI == EPI_MOO) {
+                    const double2* x = reinterpret_cast<const double2*>(a.xmoo) + row;
+                    const bool below = (c < 6) != DAG;   // S_- (lane s - 1), else S_+
+                    const bool wrap = below ? s == 0 : s == Ls - 1;
+                    const int ln = below ? (wrap ? lane0 + Ls - 1 : lane0 - 1) : (wrap ? lane0 - (Ls - 1) : lane0 + 1);
+                    const double e5 = wrap ? -a.mf * a.e : a.e;
+                    const double2 xo = x[lane0], xn = x[ln];
+                    yr = fma(sc, re[e], fma(e5, xn.x, a.d * xo.x));
+                    yi = fma(sc, im[e], fma(e5, xn.y, a.d * xo.y));
+                    if (part) nrm = fma(yr, yr, fma(yi, yi, nrm));
+                }
+                reinterpret_cast<double2*>(a.out)[row + lane0] = make_double2(yr, yi);
+            }
+        }
+        if (part) {
+            // per right-hand side, added in thread order: lanes change theirs from pass to pass
+            s_red[threadIdx.x] = nrm;
+            __syncthreads();
+            for (int r = k; r < nrhs; r += 8) {
+                double v = 0.0;
+                for (int t = j; t < 6 * 32; t += 32)
+                    if (on && lane0 / Ls == r) v += s_red[t];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+                if (j == 0) s_sum[r] += v;
+            }
+        }
+        __syncthreads();   // s_g, s_E, s_red are reused
+    }
+    if (part)
+        for (int r = threadIdx.x; r < nrhs; r += blockDim.x) a.partial[(size_t)blockIdx.x * nrhs + r] = s_sum[r];
+}
+
 // ------------------------------------------------------------- launcher
-template <class Sin, class Sout, class SL, class R, int VL, int CN5 = 0>
-static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, cudaStream_t s) {
+static HopArgs hop_args(dwf_handle* h, const HopCall& c, const TileSet& ts, bool FX) {
     const int p = c.out_parity;
-    HopArgs a;
+    HopArgs a{};
     a.in = c.in;
     a.out = c.out;
     a.xmoo = c.xmoo;
-    constexpr bool FX = std::is_same<SL, FxLink>::value;
     a.links = FX ? h->d_links_fx[p] : h->d_links[c.prec_link][p];
     a.links64 = static_cast<const double*>(h->d_links[DWF_FP64][p]);
     a.fx_info = h->d_fx_info;
@@ -1062,6 +1235,14 @@ static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, c
     a.cg_p = c.cg_p;
     a.alpha = c.alpha;
     a.run = c.run;
+    a.ntiles = ts.ntiles[p];
+    return a;
+}
+
+template <class Sin, class Sout, class SL, class R, int VL, int CN5 = 0>
+static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, cudaStream_t s) {
+    constexpr bool FX = std::is_same<SL, FxLink>::value;
+    const HopArgs a = hop_args(h, c, ts, FX);
     const int TPS = a.N5 / VL;
     // site groups per CTA: as many as fit in its threads, at most T (the
     // fixed-point hop deals sites out in turn across tiles: as many as the two
@@ -1074,9 +1255,8 @@ static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, c
     }
     int threads = (groups * TPS + 31) / 32 * 32;
     const size_t smem = hop_smem(ts.T, sizeof(SL), threads / 32, c.nrhs);
-    const int nt = ts.ntiles[p];
+    const int nt = a.ntiles;
     if (nt == 0) return DWF_OK;
-    a.ntiles = nt;
     void (*kern)(const HopArgs);
     const bool moo = c.xmoo != nullptr;
     if (c.post) {
@@ -1118,6 +1298,23 @@ static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, c
     int grid = 0;
     DWF_TRY(persistent_grid((const void*)kern, threads, smem, nt, &grid));
     kern<<<grid, threads, smem, s>>>(a);
+    note_launch();
+    DWF_CUDA(cudaGetLastError());
+    return DWF_OK;
+}
+
+// One CTA of k_hop_fx_split per tile, up to 128 lanes per SM: 8^4 x 8 (16384
+// lanes) takes 18.2 us split against 25.9, 8^4 x 16 (32768) 32.7 against 26.9.
+static bool fx_split_ok(const dwf_handle* h, const HopCall& c) {
+    return h->nsite[c.out_parity] * h->p.Ls * c.nrhs <= 152 * 128;
+}
+
+static dwf_status launch_fx_split(dwf_handle* h, const HopCall& c, const TileSet& ts, cudaStream_t s) {
+    const HopArgs a = hop_args(h, c, ts, true);
+    if (a.ntiles == 0) return DWF_OK;
+    void (*kern)(const HopArgs) = c.xmoo != nullptr ? (c.dagger ? k_hop_fx_split<true, EPI_MOO> : k_hop_fx_split<false, EPI_MOO>)
+                                                    : (c.dagger ? k_hop_fx_split<true, EPI_PLAIN> : k_hop_fx_split<false, EPI_PLAIN>);
+    kern<<<a.ntiles, 256, 0, s>>>(a);
     note_launch();
     DWF_CUDA(cudaGetLastError());
     return DWF_OK;
@@ -1217,7 +1414,8 @@ dwf_status launch_hop(dwf_handle* h, const HopCall& c, cudaStream_t s) {
     const TileSet& ts = *tsp;
     if (c.prec_link == DWF_FP64) {
         if (c.prec_in != DWF_FP64 || c.prec_out != DWF_FP64) return DWF_ERR_UNSUPPORTED;
-        if (h->fx_links) {
+        if (h->fx_links && !c.post && !c.bminv) {
+            if (fx_split_ok(h, c)) return launch_fx_split(h, c, ts, s);
             const int N5 = h->p.Ls * c.nrhs;
             if (N5 == 12) return launch_t<double, double, FxLink, double, 1, 12>(h, c, ts, s);
             if (N5 == 16) return launch_t<double, double, FxLink, double, 1, 16>(h, c, ts, s);

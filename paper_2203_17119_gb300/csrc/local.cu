@@ -14,13 +14,12 @@
 // a^k / (d (1 + mf a^Ls)) at shift distance k (a = -e/d), times -mf across
 // the wall.
 //
-// Two designs.  FP64 (k_local): each thread owns one (site, spin * colour,
-// rhs) row of Ls numbers in registers and runs the recurrences, so the
-// slow FP64 pipe does O(Ls) work per row; (d + e S_-)^-1 takes two sweeps,
-// y_0 = [x_0 - mf sum_{t>=1} a^{Ls-t} x_t] / (d (1 + mf a^Ls)), then
+// FP64 runs in local64.cu.  FP32/BF16 here: one thread per complex element
+// (k_local_sparse, k_local_dense, described below) where Ls * nrhs allows it;
+// else (k_local) each thread owns one (site, spin * colour, rhs) row of Ls
+// numbers in registers and runs the recurrences: (d + e S_-)^-1 takes two
+// sweeps, y_0 = [x_0 - mf sum_{t>=1} a^{Ls-t} x_t] / (d (1 + mf a^Ls)), then
 // y_s = (x_s - e y_{s-1}) / d, and the S_+ case the mirror image.
-// FP32/BF16 (k_local_sparse, k_local_dense): one thread per complex element,
-// described below.
 #include <algorithm>
 #include <map>
 #include <utility>
@@ -647,6 +646,23 @@ static size_t local_smem(int threads, int Ls) {
     return (size_t)4 * threads * (Ls + 1) * sizeof(R);
 }
 
+// The right-hand side counts the site-local operators take (the reductions
+// want threads of a fixed right-hand side; FP64 keeps the same limits)
+template <class R>
+static dwf_status rows_supported(int nrhs, int Ls) {
+    const int threads = local_threads<R>(nrhs);
+    if (threads < 0) {
+        set_error("local: lcm(32, nrhs=%d) exceeds 512 threads", nrhs);
+        return DWF_ERR_UNSUPPORTED;
+    }
+    const size_t smem = local_smem<R>(threads, Ls);
+    if (smem > 200 * 1024) {
+        set_error("local: %zu bytes of shared memory for nrhs=%d, Ls=%d", smem, nrhs, Ls);
+        return DWF_ERR_UNSUPPORTED;
+    }
+    return DWF_OK;
+}
+
 template <class Sin, class Sin2, class Sout, class Svec, class R, int LSM>
 static cudaError_t local_attr() {
     return cudaFuncSetAttribute(k_local<Sin, Sin2, Sout, Svec, R, LSM>,
@@ -662,7 +678,6 @@ static cudaError_t local_attr_all() {
 }
 
 dwf_status init_local_kernels() {
-    DWF_CUDA((local_attr_all<double, double, double, double, double>()));
     DWF_CUDA((local_attr_all<float, float, float, float, float>()));
     DWF_CUDA((local_attr_all<float, float, bf16, float, float>()));
     DWF_CUDA((local_attr_all<bf16, bf16, bf16, float, float>()));
@@ -674,7 +689,7 @@ dwf_status init_local_kernels() {
 template <class Sin, class Sin2, class Sout, class Svec, class R>
 static dwf_status launch_lt(dwf_handle* h, const LocalCall& c, const TileSet& ts, cudaStream_t s) {
     LocalArgs a;
-    const FiveD& f = c.f5 ? *c.f5 : h->f5[0];
+    const FiveD& f = h->f5[0];
     a.op = c.op;
     a.in = c.in;
     a.in2 = c.in2;
@@ -690,17 +705,10 @@ static dwf_status launch_lt(dwf_handle* h, const LocalCall& c, const TileSet& ts
     a.alpha = c.alpha; a.run = c.run; a.partial = c.partial;
     const int nt = ts.ntiles[c.parity];
     if (nt == 0) return DWF_OK;
-    const int threads = local_threads<R>(c.nrhs);
-    if (threads < 0) {
-        set_error("local: lcm(32, nrhs=%d) exceeds 512 threads", c.nrhs);
-        return DWF_ERR_UNSUPPORTED;
-    }
     const int Ls = h->p.Ls;
+    DWF_TRY(rows_supported<R>(c.nrhs, Ls));
+    const int threads = local_threads<R>(c.nrhs);
     const size_t smem = local_smem<R>(threads, Ls);
-    if (smem > 200 * 1024) {
-        set_error("local: %zu bytes of shared memory for nrhs=%d, Ls=%d", smem, c.nrhs, Ls);
-        return DWF_ERR_UNSUPPORTED;
-    }
     if (Ls <= 8)
         k_local<Sin, Sin2, Sout, Svec, R, 8><<<nt, threads, smem, s>>>(a);
     else if (Ls <= 16)
@@ -721,7 +729,9 @@ dwf_status launch_local(dwf_handle* h, const LocalCall& c, cudaStream_t s) {
     if (c.f5 != nullptr && (pi != DWF_FP64 || po != DWF_FP64)) return DWF_ERR_UNSUPPORTED;
     if (pi == DWF_FP64 || po == DWF_FP64) {
         if (pi != DWF_FP64 || po != DWF_FP64 || p2 != DWF_FP64) return DWF_ERR_UNSUPPORTED;
-        return launch_lt<double, double, double, double, double>(h, c, ts, s);
+        if (ts.ntiles[c.parity] == 0) return DWF_OK;
+        DWF_TRY(rows_supported<double>(c.nrhs, h->p.Ls));
+        return launch_local64(h, c, ts, s);
     }
     // FP32 arithmetic; FP32 vectors for the fused CG updates.  The matrix
     // kernel when Ls * nrhs allows a fixed rhs per thread, else the rows kernel.

@@ -22,11 +22,11 @@ namespace dwf {
 
 // Sites per tile for every kernel of an operator chain with nrhs right-hand
 // sides: the value dwf_autotune or dwf_set_tile chose (never below kMinTile),
-// else 32, whose table every handle builds when it is created.
+// else the handle's default, whose table it builds when it is created.
 int tile_for(dwf_handle* h, int nrhs) {
     auto it = h->tuned_T.find(nrhs);
     if (it != h->tuned_T.end() && it->second >= kMinTile) return it->second;
-    return 32;
+    return h->default_T;
 }
 
 // Autotuner: for each candidate (tile size, lanes per thread) time what a
@@ -37,7 +37,7 @@ int tile_for(dwf_handle* h, int nrhs) {
 // on the handle's scratch fields; keep the fastest for every kernel chain
 // with this nrhs.
 dwf_status autotune(dwf_handle* h, int nrhs, dwf_prec prec, int* best) {
-    const int cands[] = {8, 16, 32, 64, 128};
+    const int cands[] = {4, 8, 16, 32, 64, 128};
     cudaStream_t s;
     DWF_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     cudaEvent_t e0, e1;
@@ -84,6 +84,7 @@ dwf_status autotune(dwf_handle* h, int nrhs, dwf_prec prec, int* best) {
     for (int ck : chunks)
     for (int vl : vls)
     for (int T : cands) {
+        if (T < 8 && h->default_T >= 8) continue;   // tiles of 4 only where larger ones are few
         // chunked tile order only with >= 4 chunks per resident CTA (two per SM):
         // fewer leave the last round unbalanced, by more than L1 reuse gains
         if (ck > 1 && (h->nsite[0] / T) / ck < 4 * 2 * n_sm) continue;

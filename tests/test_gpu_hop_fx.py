@@ -52,7 +52,10 @@ def _check(U, psi, got, dagger):
 @pytest.mark.parametrize("dagger", [False, True])
 @pytest.mark.parametrize("dims,Ls,nrhs,span", [((4, 4, 4, 4), 8, 1, 0), ((2, 2, 2, 2), 2, 1, 6), ((6, 4, 2, 4), 12, 1, 12),
                                                ((4, 2, 6, 4), 16, 1, 3), ((4, 4, 2, 2), 6, 5, 12),
-                                               ((2, 4, 2, 2), 32, 8, 2)])
+                                               ((2, 4, 2, 2), 32, 8, 2),
+                                               # above the small-domain kernel's line
+                                               ((8, 8, 8, 8), 16, 1, 3), ((8, 6, 8, 10), 12, 1, 6),
+                                               ((8, 4, 4, 8), 12, 3, 2), ((4, 4, 4, 4), 32, 8, 1)])
 def test_uneven_neighbours(dims, Ls, nrhs, span, dagger):
     rng = np.random.default_rng(5)
     U = inputs.gauge_field(dims, "haar", rng=rng)
