@@ -258,8 +258,8 @@ __global__ void k_link_range(const double* __restrict__ l64, int64_t n /* sites 
     }
 }
 
-// Fixed-point links: w = (hi 2^32 + lo) 2^(exp - 61), lo a signed word, with
-// |w| < 2^exp.  Covered (info[1] = 1): finite links whose sizes differ by at
+// Fixed-point links: w = (hi 2^32 + lo) 2^(exp - 61), lo a signed word above
+// -2^31, with |w| < 2^exp.  Covered (info[1] = 1): finite links whose sizes differ by at
 // most 2^8, so that the common unit costs none of them precision against FP64
 // (SU(3) links lie within a factor sqrt(3)), of a size that leaves the
 // result's exponent in range.
@@ -275,7 +275,8 @@ __global__ void k_fix_links(const double* __restrict__ l64, int64_t n /* reals *
     const double scale = __hiloint2double((1023 + 61 - exp) << 20, 0);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const long long v = __double2ll_rn(l64[i] * scale);
-        fx[i] = make_int2((int)((v + (1ll << 31)) >> 32), (int)v);
+        // the low word is negated for conjugates: -2^31 becomes its neighbour (2^-61 off)
+        fx[i] = make_int2((int)((v + (1ll << 31)) >> 32), max((int)v, -2147483647));
     }
 }
 

@@ -107,3 +107,15 @@ def test_links_of_other_sizes():
     for U in (6.5 * U0, uneven, U0):
         h.set_gauge(torch.from_numpy(np.ascontiguousarray(U).reshape(-1)).cuda())
         _check(U, psi, _hop(h, psi, dims, True), True)
+
+
+def test_links_whose_low_word_is_the_lowest():
+    """Imaginary parts (2 m + 1) 2^-30: a fixed-point low word of exactly -2^31,
+    whose negative is not a 32-bit number."""
+    dims, Ls = (4, 4, 2, 4), 8
+    rng = np.random.default_rng(9)
+    U = inputs.gauge_field(dims, "exp", rng=rng)
+    m = rng.integers(-2 ** 27, 2 ** 27, U.shape)
+    U = 0.9 * U.real + 1j * np.ldexp(2.0 * m + 1.0, -30)
+    psi = [inputs.gaussian_source(dims, Ls, rng=rng)]
+    _check(U, psi, _hop(_handle(dims, Ls, U), psi, dims, False), False)
