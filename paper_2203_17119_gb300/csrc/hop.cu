@@ -26,6 +26,7 @@
 #include "dwf_internal.cuh"
 
 namespace dwf {
+
 struct HopArgs {
     const void* in;
     void* out;
@@ -37,6 +38,7 @@ struct HopArgs {
     const int* nbr;      // [site][8]
     const int4* tiles;
     int T, N5, Ls, nrhs, ntiles;
+    int deal;            // sites are dealt to the site groups in turn across tiles
     int chunk;           // consecutive tiles a CTA takes before striding: neighbouring rows of
                          // the lattice on one SM, so y-neighbours are re-read from L1
     double scale, d, e, mf, b5, c5;
@@ -793,42 +795,53 @@ __device__ __forceinline__ double hop_store(const HopArgs& a, int N5, int64_t si
     const R f_above = hi_wrap ? -mf : (R)1;
     double nrm = 0.0;
     float nrm_f = 0.f;
+    // FP32: four rows at a time, their loads in flight before the first store
+    // (one at a time, each row waited out its own latency: 791 us at 32^4 x 16
+    // against 710, the plain epilogue 519; six rows gain nothing more).  FP64 has
+    // no registers for more than one row.
+    constexpr int NB = sizeof(R) == 8 ? 1 : 4;
 #pragma unroll
-    for (int c = 0; c < 12; ++c) {
-        R xr[VL], xi[VL];
-        load_lanes<Sout, VL, R>(xb + (int64_t)(c * N5 + lane0) * 2, xr, xi);
-        // upper spins use S_- (x_{s-1}) unless dagger, lower S_+
-        const bool use_below = (c < 6) != DAG;
-        R nr, ni, fn;
-        if constexpr (kLaneShfl<VL, CN5>) {
-            // the neighbouring lane is held by the adjacent thread of the site group
-            nr = __shfl_sync(nb.mask, use_below ? xr[VL - 1] : xr[0], use_below ? nb.src_dn : nb.src_up);
-            ni = __shfl_sync(nb.mask, use_below ? xi[VL - 1] : xi[0], use_below ? nb.src_dn : nb.src_up);
-            if constexpr (sizeof(R) == 8) fn = use_below ? f_below : f_above;   // (nb's factors are FP32)
-            else fn = (R)(use_below ? nb.f_dn : nb.f_up);
-        } else {
-            load_c1<Sout, R>(xb + (int64_t)(c * N5 + (use_below ? l_below : l_above)) * 2, nr, ni);
-            fn = use_below ? f_below : f_above;
+    for (int c0 = 0; c0 < 12; c0 += NB) {
+        R xr[NB][VL], xi[NB][VL], nr[NB], ni[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            const int c = c0 + b;
+            load_lanes<Sout, VL, R>(xb + (int64_t)(c * N5 + lane0) * 2, xr[b], xi[b]);
+            // upper spins use S_- (x_{s-1}) unless dagger, lower S_+
+            if constexpr (!kLaneShfl<VL, CN5>)
+                load_c1<Sout, R>(xb + (int64_t)(c * N5 + ((c < 6) != DAG ? l_below : l_above)) * 2, nr[b], ni[b]);
         }
-        R orr[VL], oi[VL];
-        float part = 0.f;
 #pragma unroll
-        for (int v = 0; v < VL; ++v) {
-            R sr, si;
-            if (use_below) {
-                sr = (v == 0) ? fn * nr : xr[v - 1];
-                si = (v == 0) ? fn * ni : xi[v - 1];
-            } else {
-                sr = (v == VL - 1) ? fn * nr : xr[(v + 1) % VL];
-                si = (v == VL - 1) ? fn * ni : xi[(v + 1) % VL];
+        for (int b = 0; b < NB; ++b) {
+            const int c = c0 + b;
+            const bool use_below = (c < 6) != DAG;
+            R fn = use_below ? f_below : f_above;
+            if constexpr (kLaneShfl<VL, CN5>) {
+                // the neighbouring lane is held by the adjacent thread of the site group
+                nr[b] = __shfl_sync(nb.mask, use_below ? xr[b][VL - 1] : xr[b][0], use_below ? nb.src_dn : nb.src_up);
+                ni[b] = __shfl_sync(nb.mask, use_below ? xi[b][VL - 1] : xi[b][0], use_below ? nb.src_dn : nb.src_up);
+                if constexpr (sizeof(R) == 4) fn = (R)(use_below ? nb.f_dn : nb.f_up);   // (nb's factors are FP32)
             }
-            orr[v] = d * xr[v] + e * sr + sc * ar[c][v];
-            oi[v] = d * xi[v] + e * si + sc * ai[c][v];
-            part += (float)(orr[v] * orr[v] + oi[v] * oi[v]);
-            if (sizeof(R) == 8 && a.partial != nullptr) nrm += (double)orr[v] * orr[v] + (double)oi[v] * oi[v];
+            R orr[VL], oi[VL];
+            float part = 0.f;
+#pragma unroll
+            for (int v = 0; v < VL; ++v) {
+                R sr, si;
+                if (use_below) {
+                    sr = (v == 0) ? fn * nr[b] : xr[b][v - 1];
+                    si = (v == 0) ? fn * ni[b] : xi[b][v - 1];
+                } else {
+                    sr = (v == VL - 1) ? fn * nr[b] : xr[b][(v + 1) % VL];
+                    si = (v == VL - 1) ? fn * ni[b] : xi[b][(v + 1) % VL];
+                }
+                orr[v] = d * xr[b][v] + e * sr + sc * ar[c][v];
+                oi[v] = d * xi[b][v] + e * si + sc * ai[c][v];
+                part += (float)(orr[v] * orr[v] + oi[v] * oi[v]);
+                if (sizeof(R) == 8 && a.partial != nullptr) nrm += (double)orr[v] * orr[v] + (double)oi[v] * oi[v];
+            }
+            if (sizeof(R) != 8) nrm_f += part;
+            store_lanes<Sout, VL, R, true>(out + (int64_t)c * N5 * 2, orr, oi);
         }
-        if (sizeof(R) != 8) nrm_f += part;
-        store_lanes<Sout, VL, R, true>(out + (int64_t)c * N5 * 2, orr, oi);
     }
     return sizeof(R) == 8 ? nrm : (double)nrm_f;
 }
@@ -946,8 +959,8 @@ k_hop(const HopArgs a) {
 
     int k = 0;
     const int2 fx_info = FX ? *reinterpret_cast<const int2*>(a.fx_info) : make_int2(0, 0);
-    int turn = 0;   // fixed-point hop: sites done so far mod G, so that the groups that
-                    // take a tile's remainder change from tile to tile
+    int turn = 0;   // a.deal: sites done so far mod G, so that the groups that take a tile's
+                    // remainder change from tile to tile
     for (int tile = tile_of(0); tile < nt; tile = tile_of(++k)) {
         const int b = k & 1;
         const uint32_t ph = (uint32_t)((k >> 1) & 1);
@@ -965,7 +978,7 @@ k_hop(const HopArgs a) {
         const int* s_nbr_t = reinterpret_cast<const int*>(smem + b * buf_bytes + link_bytes);
         double tile_norm = 0.0;
         int first = sg;
-        if constexpr (FX) {
+        if (a.deal) {
             first = sg - turn + (sg < turn ? G : 0);
             turn = (turn + count) % G;
         }
@@ -1242,17 +1255,21 @@ static HopArgs hop_args(dwf_handle* h, const HopCall& c, const TileSet& ts, bool
 template <class Sin, class Sout, class SL, class R, int VL, int CN5 = 0>
 static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, cudaStream_t s) {
     constexpr bool FX = std::is_same<SL, FxLink>::value;
-    const HopArgs a = hop_args(h, c, ts, FX);
+    HopArgs a = hop_args(h, c, ts, FX);
     const int TPS = a.N5 / VL;
-    // site groups per CTA: as many as fit in its threads, at most T (the
-    // fixed-point hop deals sites out in turn across tiles: as many as the two
-    // buffered tiles hold)
+    // site groups per CTA: as many as fit in its threads, at most T (fixed-point
+    // hop: at most what the two buffered tiles hold, where a CTA gets several).
+    // Where they do not divide T, sites are dealt out in turn across tiles: at
+    // 16^4 x 12 with 3 right-hand sides 95.7 -> 87.0 us.  (More groups than T in
+    // FP32 lost 1 to 6% at 16^4 x 10 and 16^4 x 12.)
     int groups = kHopThreads<SL> / TPS;
-    if (groups > (FX ? 2 : 1) * ts.T) groups = (FX ? 2 : 1) * ts.T;
+    const int most = FX && a.ntiles > 2 * 152 ? 2 * ts.T : ts.T;
+    if (groups > most) groups = most;
     if (groups < 1) {
         set_error("hop: %d threads per site exceed %d", TPS, kHopThreads<SL>);
         return DWF_ERR_ARG;
     }
+    a.deal = ts.T % groups != 0;
     int threads = (groups * TPS + 31) / 32 * 32;
     const size_t smem = hop_smem(ts.T, sizeof(SL), threads / 32, c.nrhs);
     const int nt = a.ntiles;
