@@ -602,7 +602,7 @@ dwf_status dwf_one_flavour_heatbath(dwf_handle* h, dwf_handle* hd, double* phi, 
  * cosh(order arccosh z).  Three-term recurrence, `order` applications of A.
  * in, out: distinct odd cb fields of precision `prec` (FP64 or FP32, which is
  * also the operator's), nrhs right-hand sides.  Errors: DWF_ERR_ARG for
- * order < 0, hi <= lo or another precision.  Allocates three cb fields for
+ * order < 0, hi <= lo or another precision.  Allocates two cb fields for
  * the call and ends with a stream sync. */
 dwf_status dwf_chebyshev_filter(dwf_handle* h, void* out, const void* in, int order, double lo, double hi,
                                 dwf_prec prec, int nrhs, void* stream);

@@ -315,6 +315,15 @@ dwf_status multishift_solve(dwf_handle* h, double* x, const double* b, const dou
                             int nshift, int nrhs, const dwf_solver_params* sp,
                             dwf_solver_stats* stats, cudaStream_t s);
 
+// L_POST: result = a * result + bu * u + bv * v (fields of the result's precision; v may be the output)
+struct LinComb {
+    double a;
+    const void* u;
+    double bu;
+    const void* v;
+    double bv;
+};
+
 struct LocalCall {
     LocalOp op;
     const void* in;          // field of prec_in
@@ -332,6 +341,7 @@ struct LocalCall {
     double* partial;         // per tile, per rhs |result|^2 (nullable)
     int T;
     const FiveD* f5 = nullptr;   // FP64 only: fifth-dimension coefficients other than the handle's
+    const LinComb* lin = nullptr;   // L_POST without a CG update
 };
 dwf_status launch_local(dwf_handle* h, const LocalCall& c, cudaStream_t s);
 dwf_status launch_local64(dwf_handle* h, const LocalCall& c, const TileSet& ts, cudaStream_t s);   // FP64
@@ -371,7 +381,7 @@ dwf_status op_dslash_eo(dwf_handle* h, void* out, const void* in, int p, int dag
                         dwf_prec prec, int nrhs, void* tmp, cudaStream_t s);
 dwf_status op_mpc(dwf_handle* h, void* out, const void* in, int dagger, dwf_prec pv, dwf_prec po,
                   int nrhs, void* tmpA, void* tmpB, double* partial, const CgFuse* cg,
-                  cudaStream_t s);
+                  cudaStream_t s, const LinComb* lin = nullptr);   // lin: dagger only
 dwf_status op_apply_d(dwf_handle* h, void* out, const void* in, int dagger, dwf_prec prec,
                       int nrhs, void* tmp, cudaStream_t s);
 dwf_status op_mpc_pre(dwf_handle* h, void* out, const void* p, const void* t1, dwf_prec pv,

@@ -42,8 +42,9 @@ struct LocalArgs {
     const int4* tiles;
     int Ls, nrhs, dagger;
     int rows_warp, rows_block;   // rows a warp and a block take at a time (the latter a multiple of nrhs)
-    float c0, c1;                // out = c0 x + c1 S x (of w for the inverse)
-    float z0, z1;                // L_POST: + z0 z + z1 S z
+    float scale;
+    float c0, c1;                // out = scale (c0 x + c1 S x) (the inverse: of w, scale folded in)
+    float z0, z1;                // L_POST: out = c0 x + c1 S x + scale (z0 z + z1 S z)
     float mf;
     float a, wall;               // inverse: a, mf / (1 + mf a^Ls)
     float* cg_x;
@@ -52,6 +53,9 @@ struct LocalArgs {
     const double* alpha;
     const int* run;
     double* partial;
+    const void* lin_u;           // L_POST: out = lin_a out + lin_bu u + lin_bv v
+    const void* lin_v;
+    float lin_a, lin_bu, lin_bv;
 };
 
 enum { K_ONE = 0, K_POST = 1, K_PB = 2, K_INV = 3 };
@@ -64,15 +68,17 @@ struct RowPos {
     float f_dn, f_up;
 };
 
-// S x for the thread's lanes, S_- (down) or S_+
+// y = c0 x + c1 S x on the thread's lanes, S_- (down) or S_+
 template <int VL>
-__device__ __forceinline__ void shift_row(const float (&x)[VL], float (&y)[VL], bool down, const RowPos& p) {
-    const float nb = __shfl_sync(0xffffffffu, down ? x[VL - 1] : x[0], down ? p.src_dn : p.src_up) *
-                     (down ? p.f_dn : p.f_up);
+__device__ __forceinline__ void shift_sum(float c0, float c1, const float (&x)[VL], float (&y)[VL], bool down,
+                                          const RowPos& p) {
+    const float nb = __shfl_sync(0xffffffffu, down ? x[VL - 1] : x[0], down ? p.src_dn : p.src_up);
+    const float cw = c1 * (down ? p.f_dn : p.f_up);   // of the lane whose neighbour is another thread's
 #pragma unroll
     for (int v = 0; v < VL; ++v) {
         const float lo = v > 0 ? x[v > 0 ? v - 1 : 0] : nb, hi = v < VL - 1 ? x[v < VL - 1 ? v + 1 : 0] : nb;
-        y[v] = down ? lo : hi;
+        const bool edge = down ? v == 0 : v == VL - 1;
+        y[v] = fmaf(edge ? cw : c1, down ? lo : hi, c0 * x[v]);
     }
 }
 
@@ -192,21 +198,18 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
 #pragma unroll
                 for (int v = 0; v < VL; ++v) { yr[v] = a.c0 * xr[u][v]; yi[v] = a.c0 * xi[u][v]; }
             } else {
-                shift_row<VL>(xr[u], tr, down, rp);
-                shift_row<VL>(xi[u], ti, down, rp);
-#pragma unroll
-                for (int v = 0; v < VL; ++v) {
-                    yr[v] = fmaf(a.c1, tr[v], a.c0 * xr[u][v]);
-                    yi[v] = fmaf(a.c1, ti[v], a.c0 * xi[u][v]);
-                }
+                shift_sum<VL>(a.c0, a.c1, xr[u], yr, down, rp);
+                shift_sum<VL>(a.c0, a.c1, xi[u], yi, down, rp);
             }
             if (KIND == K_POST) {
-                shift_row<VL>(zr[u], tr, down, rp);
-                shift_row<VL>(zi[u], ti, down, rp);
+                shift_sum<VL>(a.z0, a.z1, zr[u], tr, down, rp);
+                shift_sum<VL>(a.z0, a.z1, zi[u], ti, down, rp);
+            }
+            if (KIND == K_ONE || KIND == K_POST || KIND == K_PB) {
 #pragma unroll
                 for (int v = 0; v < VL; ++v) {
-                    yr[v] = fmaf(a.z0, zr[u][v], fmaf(a.z1, tr[v], yr[v]));
-                    yi[v] = fmaf(a.z0, zi[u][v], fmaf(a.z1, ti[v], yi[v]));
+                    yr[v] = KIND == K_POST ? fmaf(a.scale, tr[v], yr[v]) : a.scale * yr[v];
+                    yi[v] = KIND == K_POST ? fmaf(a.scale, ti[v], yi[v]) : a.scale * yi[v];
                 }
             }
             if (!ok) continue;
@@ -230,6 +233,19 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
 #pragma unroll
                 for (int v = 0; v < VL; ++v) { yr[v] = rr[v]; yi[v] = ri[v]; }
             } else if (a.out != nullptr) {
+                if (KIND == K_POST && a.lin_u != nullptr) {
+                    float ur[VL], ui[VL], vr[VL], vi[VL];
+#pragma unroll
+                    for (int v = 0; v < VL; ++v) vr[v] = vi[v] = 0.f;
+                    load_lanes<Sout, VL, float>(reinterpret_cast<const Sout*>(a.lin_u) + 2 * g, ur, ui);
+                    if (a.lin_v != nullptr)
+                        load_lanes<Sout, VL, float>(reinterpret_cast<const Sout*>(a.lin_v) + 2 * g, vr, vi);
+#pragma unroll
+                    for (int v = 0; v < VL; ++v) {
+                        yr[v] = fmaf(a.lin_a, yr[v], fmaf(a.lin_bu, ur[v], a.lin_bv * vr[v]));
+                        yi[v] = fmaf(a.lin_a, yi[v], fmaf(a.lin_bu, ui[v], a.lin_bv * vi[v]));
+                    }
+                }
                 store_lanes<Sout, VL, float>(reinterpret_cast<Sout*>(a.out) + 2 * g, yr, yi);
             }
 #pragma unroll
@@ -264,6 +280,7 @@ static dwf_status launch_vl(dwf_handle* h, const LocalCall& c, const TileSet& ts
         return DWF_ERR_UNSUPPORTED;
     }
     a.mf = (float)f.mf;
+    a.scale = (float)c.scale;
     a.cg_x = (float*)c.cg_x;
     a.cg_r = (float*)c.cg_r;
     a.cg_p = (float*)const_cast<void*>(c.cg_p);
@@ -286,18 +303,25 @@ static dwf_status launch_vl(dwf_handle* h, const LocalCall& c, const TileSet& ts
         case L_POST:
             a.c0 = (float)f.d;
             a.c1 = (float)f.e;
-            a.z0 = (float)(c.scale * f.b5);
-            a.z1 = (float)(c.scale * f.c5);
+            a.z0 = (float)f.b5;
+            a.z1 = (float)f.c5;
+            if (c.lin) {
+                a.lin_u = c.lin->u;
+                a.lin_v = c.lin->bv != 0.0 ? c.lin->v : nullptr;
+                a.lin_a = (float)c.lin->a;
+                a.lin_bu = (float)c.lin->bu;
+                a.lin_bv = (float)c.lin->bv;
+            }
             kern = k_local<Sin, Sin2, Sout, VL, K_POST>;
             break;
         case L_PB:
-            a.c0 = (float)(c.scale * f.b5);
-            a.c1 = (float)(c.scale * f.c5);
+            a.c0 = (float)f.b5;
+            a.c1 = (float)f.c5;
             kern = k_local<Sin, Sin2, Sout, VL, K_PB>;
             break;
         default:
-            a.c0 = (float)(c.scale * (c.op == L_MOOEE ? f.d : c.op == L_B ? f.b5 : 1.0));
-            a.c1 = (float)(c.scale * (c.op == L_MOOEE ? f.e : c.op == L_B ? f.c5 : 0.0));
+            a.c0 = (float)(c.op == L_MOOEE ? f.d : c.op == L_B ? f.b5 : 1.0);
+            a.c1 = (float)(c.op == L_MOOEE ? f.e : c.op == L_B ? f.c5 : 0.0);
     }
     kern<<<nt, kLocalThreads, 0, s>>>(a);
     note_launch();

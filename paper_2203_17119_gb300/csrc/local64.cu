@@ -45,6 +45,9 @@ struct Local64Args {
     const double* alpha;
     const int* run;
     double* partial;
+    const double2* lin_u;   // L_POST: out = lin_a out + lin_bu u + lin_bv v
+    const double2* lin_v;
+    double lin_a, lin_bu, lin_bv;
 };
 
 constexpr int kL64Ept = 2;   // elements per thread and chunk
@@ -129,6 +132,11 @@ __global__ void __launch_bounds__(256) k_local64(const Local64Args a) {
                 yr = r.x;
                 yi = r.y;
             } else if (a.out != nullptr) {
+                if (KIND == L64_POST && a.lin_u != nullptr) {
+                    const double2 u = a.lin_u[g], v = a.lin_v != nullptr ? a.lin_v[g] : make_double2(0.0, 0.0);
+                    yr = fma(a.lin_a, yr, fma(a.lin_bu, u.x, a.lin_bv * v.x));
+                    yi = fma(a.lin_a, yi, fma(a.lin_bu, u.y, a.lin_bv * v.y));
+                }
                 a.out[g] = make_double2(yr, yi);
             }
             if (a.partial) nrm = fma(yr, yr, fma(yi, yi, nrm));
@@ -242,6 +250,13 @@ dwf_status launch_local64(dwf_handle* h, const LocalCall& c, const TileSet& ts, 
                 a.c1 = f.e;
                 a.z0 = c.scale * f.b5;
                 a.z1 = c.scale * f.c5;
+                if (c.lin) {
+                    a.lin_u = (const double2*)c.lin->u;
+                    a.lin_v = c.lin->bv != 0.0 ? (const double2*)c.lin->v : nullptr;
+                    a.lin_a = c.lin->a;
+                    a.lin_bu = c.lin->bu;
+                    a.lin_bv = c.lin->bv;
+                }
                 k_local64<L64_POST><<<nt, threads, 2 * plane, s>>>(a);
                 break;
             case L_PB:

@@ -348,10 +348,11 @@ static dwf_status hop_then_bminv(dwf_handle* h, const void* in, int dagger, dwf_
 // the CG vectors), po: operator precision (links and intermediates).
 // tmpA/tmpB: cb temporaries of precision po.  partial: per-tile |out|^2.
 // cg: optional fused CG step of the adjoint (x += alpha p, r -= alpha out).
+// lin: optional linear combination of the adjoint's result (out = a out + bu u + bv v).
 
 dwf_status op_mpc(dwf_handle* h, void* out, const void* in, int dagger, dwf_prec pv, dwf_prec po,
                   int nrhs, void* tmpA, void* tmpB, double* partial, const CgFuse* cg,
-                  cudaStream_t s) {
+                  cudaStream_t s, const LinComb* lin) {
     const double b5 = h->p.b5;
     if (!dagger) {
         const void* src = in;
@@ -396,6 +397,7 @@ dwf_status op_mpc(dwf_handle* h, void* out, const void* in, int dagger, dwf_prec
     c.scale = -0.25;
     c.partial = partial;
     c.T = tileT(h, 0, pv == DWF_FP64 ? DWF_FP64 : DWF_FP32, nrhs);
+    c.lin = lin;
     if (cg) {
         c.cg_x = cg->x;
         c.cg_r = cg->r;
