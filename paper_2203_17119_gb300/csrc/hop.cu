@@ -38,6 +38,7 @@ struct HopArgs {
     const int* nbr;      // [site][8]
     const int4* tiles;
     int T, N5, Ls, nrhs, ntiles;
+    int lane_chunk;      // lanes of a site a CTA takes at a time (N5, or whole right-hand sides dividing it)
     int deal;            // sites are dealt to the site groups in turn across tiles
     int chunk;           // consecutive tiles a CTA takes before striding: neighbouring rows of
                          // the lattice on one SM, so y-neighbours are re-read from L1
@@ -869,7 +870,9 @@ k_hop(const HopArgs a) {
     constexpr bool FX = std::is_same<SL, FxLink>::value;
     extern __shared__ __align__(128) unsigned char smem[];
     const int N5 = CN5 > 0 ? CN5 : a.N5;
-    const int TPS = N5 / VL;
+    const int LC = CN5 > 0 ? CN5 : a.lane_chunk;   // lanes of a site this CTA takes, from lc
+    const int lc = CN5 > 0 ? 0 : (int)blockIdx.y * LC;
+    const int TPS = LC / VL;
     const size_t link_bytes = (size_t)a.T * 144 * sizeof(SL);
     const size_t buf_bytes = link_bytes + (size_t)a.T * 32;
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 2 * buf_bytes);
@@ -905,8 +908,9 @@ k_hop(const HopArgs a) {
 
     const int G = blockDim.x / TPS;
     const int sg = threadIdx.x / TPS;
-    const int lane0 = (threadIdx.x - sg * TPS) * VL;
+    const int lane0 = lc + (threadIdx.x - sg * TPS) * VL;
     const int rhs = lane0 / a.Ls;   // of this thread's lanes (threads without sites add 0)
+    const int rhs0 = lc / a.Ls, rhs1 = (lc + LC) / a.Ls;
     const bool part = (EPI == EPI_MOO || EPI == EPI_POST) && a.partial != nullptr;
     ScanCtx<VL> sk{};
     if constexpr (EPI == EPI_BMINV) {
@@ -944,14 +948,14 @@ k_hop(const HopArgs a) {
     if constexpr (EPI == EPI_POST || (EPI == EPI_MOO && kLaneShfl<VL, CN5>)) {
         // site groups are warp-aligned here (TPS divides 32, checked on the host)
         const int wl = threadIdx.x & 31;
-        const int tig = lane0 / VL;
+        const int tig = (lane0 - lc) / VL;
         const int gb = wl - tig;
         const int s_first = lane0 % a.Ls, s_last = (lane0 + VL - 1) % a.Ls;
         const int rb = lane0 - s_first;
         const int above = s_last == a.Ls - 1 ? rb : lane0 + VL;
         const int below = s_first == 0 ? rb + a.Ls - 1 : lane0 - 1;
-        nbrs.src_up = gb + above / VL;
-        nbrs.src_dn = gb + below / VL;
+        nbrs.src_up = gb + (above - lc) / VL;
+        nbrs.src_dn = gb + (below - lc) / VL;
         nbrs.f_up = s_last == a.Ls - 1 ? -(float)a.mf : 1.f;
         nbrs.f_dn = s_first == 0 ? -(float)a.mf : 1.f;
         nbrs.mask = TPS >= 32 ? 0xffffffffu : (((1u << TPS) - 1u) << gb);
@@ -976,6 +980,7 @@ k_hop(const HopArgs a) {
         const int begin = tl.y, count = tl.z;
         const SL* s_link_t = reinterpret_cast<const SL*>(smem + b * buf_bytes);
         const int* s_nbr_t = reinterpret_cast<const int*>(smem + b * buf_bytes + link_bytes);
+        double* red = s_red + (size_t)b * nwarps * a.nrhs;
         double tile_norm = 0.0;
         int first = sg;
         if (a.deal) {
@@ -1039,9 +1044,8 @@ k_hop(const HopArgs a) {
             }
             tile_norm += hop_store<Sout, R, VL, DAG, EPI, CN5>(a, N5, begin + sl, lane0, ar, ai, factor, nbrs, tl.x, sk);
         }
-        double* red = s_red + (size_t)b * nwarps * a.nrhs;
         if (part) {
-            for (int r = 0; r < a.nrhs; ++r) {
+            for (int r = rhs0; r < rhs1; ++r) {
                 double v = rhs == r ? tile_norm : 0.0;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -1054,7 +1058,7 @@ k_hop(const HopArgs a) {
             if (atomicAdd(&done[b], 1) == nwarps - 1) {   // the last warp out
                 __threadfence_block();
                 if (part)
-                    for (int r = 0; r < a.nrhs; ++r) {
+                    for (int r = rhs0; r < rhs1; ++r) {
                         double sum = 0.0;
                         for (int w = 0; w < nwarps; ++w) sum += red[w * a.nrhs + r];
                         a.partial[(size_t)tile * a.nrhs + r] = sum;
@@ -1252,11 +1256,30 @@ static HopArgs hop_args(dwf_handle* h, const HopCall& c, const TileSet& ts, bool
     return a;
 }
 
+// Lanes of a site that a CTA takes: all of them, or, with many right-hand
+// sides, whole right-hand sides of at most 32 lanes whose threads divide a
+// warp (the chunks side by side in the grid), so that a CTA's pass covers a
+// row of neighbouring sites that it finds in L1 again; with 256 lanes a pass is
+// two sites, 24 KB a row.  Bare hop, whole / chunked, Ls = 16: FP32 12^4 with 16
+// right-hand sides 302 / 160 us, 16^4 with 8 305 / 262, 12^4 with 3 49.3 / 45.5;
+// 8^4 with 16 (0.5 M lanes) 35.8 / 37.9, so not on small domains; FP64 12^4 with
+// 16 1851 / 1406, but with 16-lane chunks 2260; BF16 12^4 with 16 217 / 158, with
+// 3 46.2 / 42.8, but 16^4 with 8 232 / 240 (its 128 lanes are 512 bytes).
+static int lane_chunk(int Ls, int nrhs, int VL, dwf_prec link, int64_t nsite) {
+    const int N5 = Ls * nrhs;
+    if (N5 <= 32 || nsite * N5 < (link == DWF_FP64 ? 0 : 1 << 20)) return N5;
+    if (link == DWF_BF16 && N5 > 64 && N5 <= 128) return N5;
+    for (int k = 32 / Ls; k >= 1; --k)
+        if (nrhs % k == 0 && 32 % (k * Ls / VL) == 0 && (link != DWF_FP64 || k * Ls == 32)) return k * Ls;
+    return N5;
+}
+
 template <class Sin, class Sout, class SL, class R, int VL, int CN5 = 0>
 static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, cudaStream_t s) {
     constexpr bool FX = std::is_same<SL, FxLink>::value;
     HopArgs a = hop_args(h, c, ts, FX);
-    const int TPS = a.N5 / VL;
+    a.lane_chunk = CN5 > 0 || c.post || c.bminv ? a.N5 : lane_chunk(h->p.Ls, c.nrhs, VL, c.prec_link, h->nsite[c.out_parity]);
+    const int TPS = a.lane_chunk / VL;
     // site groups per CTA: as many as fit in its threads, at most T (fixed-point
     // hop: at most what the two buffered tiles hold, where a CTA gets several).
     // Where they do not divide T, sites are dealt out in turn across tiles: at
@@ -1313,8 +1336,9 @@ static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, c
     }
     // persistent grid: as many CTAs as are resident at once, at most one per tile
     int grid = 0;
-    DWF_TRY(persistent_grid((const void*)kern, threads, smem, nt, &grid));
-    kern<<<grid, threads, smem, s>>>(a);
+    const int chunks = a.N5 / a.lane_chunk;
+    DWF_TRY(persistent_grid((const void*)kern, threads, smem, nt * chunks, &grid));
+    kern<<<dim3((grid + chunks - 1) / chunks, chunks), threads, smem, s>>>(a);
     note_launch();
     DWF_CUDA(cudaGetLastError());
     return DWF_OK;

@@ -119,3 +119,27 @@ def test_links_whose_low_word_is_the_lowest():
     U = 0.9 * U.real + 1j * np.ldexp(2.0 * m + 1.0, -30)
     psi = [inputs.gaussian_source(dims, Ls, rng=rng)]
     _check(U, psi, _hop(_handle(dims, Ls, U), psi, dims, False), False)
+
+
+@pytest.mark.parametrize("dims,nrhs,inner", [((6, 6, 6, 6), 4, G.FP64), ((12, 8, 8, 12), 16, G.FP32)])
+def test_solves_with_lanes_in_chunks(dims, nrhs, inner):
+    """Many right-hand sides go through the hop in chunks of 32 lanes, each with
+    its own part of the per-tile norms: every system of a batched solve (Ls = 16)
+    reaches its tolerance, and the first equals its solve alone."""
+    Ls, tol = 16, 1e-11
+    rng = np.random.default_rng(10)
+    U = torch.from_numpy(inputs.gauge_field(dims, "exp", rng=rng).reshape(-1)).cuda()
+    act = G.Action(1.8, 0.05, 1.5, 0.5)
+    h, h1 = G.Handle(dims, Ls, act, nrhs_max=nrhs), G.Handle(dims, Ls, act)
+    h.set_gauge(U)
+    h1.set_gauge(U)
+    b = torch.randn(h.full_shape(nrhs), dtype=torch.float64, device="cuda",
+                    generator=torch.Generator(device="cuda").manual_seed(11))
+    x = torch.zeros_like(b)
+    stats, rc = h.cgne_solve(x, b, nrhs=nrhs, tol=tol, inner=inner)
+    assert rc == 0 and all(st["true_resid"] <= tol for st in stats)
+    b1 = b[:, :, :1].contiguous()
+    x1 = torch.zeros_like(b1)
+    h1.cgne_solve(x1, b1, tol=tol, inner=inner)
+    # both within tol of the residual: the condition of D (below 1e2 here) times tol, doubled
+    assert float((x[:, :, :1] - x1).norm() / x1.norm()) <= 2e2 * tol
