@@ -389,7 +389,7 @@ __device__ __forceinline__ void hop_dir(const Sin* __restrict__ in, const int* s
 // arithmetic comes out no larger than the FP64 form's.  Lanes the fixed point
 // does not cover -- a NaN, an infinity, all components below 2^-895 or one
 // above 2^56 -- run the FP64 form; so does a handle whose links differ in size
-// by more than 2^8 (set_gauge).  Measured, bare hop: 16^4 x 12 650 -> 205 us,
+// by more than 2^8 (set_gauge).  Measured, bare hop: 16^4 x 12 650 -> 209 us,
 // 24^4 x 16 4.17 -> 1.34 ms (FP64 form -> this); no pipe is full (FP64 half,
 // integer multiply-add about 60%): the chains of dependent integer
 // instructions at 16 warps per SM are what is left.
@@ -1280,13 +1280,16 @@ static dwf_status launch_t(dwf_handle* h, const HopCall& c, const TileSet& ts, c
     HopArgs a = hop_args(h, c, ts, FX);
     a.lane_chunk = CN5 > 0 || c.post || c.bminv ? a.N5 : lane_chunk(h->p.Ls, c.nrhs, VL, c.prec_link, h->nsite[c.out_parity]);
     const int TPS = a.lane_chunk / VL;
-    // site groups per CTA: as many as fit in its threads, at most T (fixed-point
-    // hop: at most what the two buffered tiles hold, where a CTA gets several).
+    // site groups per CTA: as many as fit in its threads, at most T.  Fixed-point
+    // hop, where T groups are fewer than 384 threads and a CTA gets several
+    // tiles: as many as the two buffered tiles hold (T / 2 T groups: 16^4 x 10
+    // 223 / 198 us, 16^4 x 6 134 / 122; but 16^4 x 12, 384 threads, 211 / 228, and
+    // with two tiles per CTA 10^4 x 16 59 / 65, 10^4 x 12 53 / 56).
     // Where they do not divide T, sites are dealt out in turn across tiles: at
     // 16^4 x 12 with 3 right-hand sides 95.7 -> 87.0 us.  (More groups than T in
     // FP32 lost 1 to 6% at 16^4 x 10 and 16^4 x 12.)
     int groups = kHopThreads<SL> / TPS;
-    const int most = FX && a.ntiles > 2 * 152 ? 2 * ts.T : ts.T;
+    const int most = FX && a.ntiles > 4 * 152 && ts.T * TPS < 384 ? 2 * ts.T : ts.T;
     if (groups > most) groups = most;
     if (groups < 1) {
         set_error("hop: %d threads per site exceed %d", TPS, kHopThreads<SL>);
