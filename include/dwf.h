@@ -160,7 +160,8 @@ dwf_status dwf_box_sites(const dwf_handle* h, int box, int parity,
 /* Load the gauge field (device pointer, canonical complex128 layout of the
  * whole lattice, read during the call only).  Builds the FP64/FP32/BF16
  * per-parity link tables (forward U_mu(x) and backward U_mu(x-mu)^+ per
- * site, zero for links cut by the domain); ends with a stream sync. */
+ * site, zero for links cut by the domain) and the fixed-point form of the
+ * FP64 table that the FP64 hop reads; ends with a stream sync. */
 dwf_status dwf_set_gauge(dwf_handle* h, const double* U, void* stream);
 
 /* canonical complex128 <-> full field of precision `prec` (layout kernels). */

@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(256) k_odd_sum(const OddArgs a) {
 // next 32 pixels are loaded into registers during the arithmetic.  One thread
 // per pair reading scalars from the fields' own order over both parities ran
 // at 7 TFLOP/s (29.8 ms each of the two gradients); the whole training step of
-// batch 4 at 16^4 x 12 went from 80.5 to 18.3 ms with this kernel and the
+// batch 4 at 16^4 x 12 went from 80.2 to 17.9 ms with this kernel and the
 // zero directions left out of the mixes.
 constexpr int kWgThreads = 256;
 constexpr int kWgPix = 32;
