@@ -22,13 +22,18 @@
 //   w_s = P_s - mf / (1 + mf a^Ls) a^(s+1) P_(Ls-1),
 // P in the thread first, then across threads (Hillis-Steele with factors
 // a^VL, a^2VL, ...); S_+ is the mirror image, so rows of either chirality run
-// the same code on mirrored lanes.
+// the same code on mirrored lanes.  For |a| > 1 (c5 well above b5) P grows like
+// |a|^Ls and the wall term would have to cancel it (FP32 at b5 = 1, c5 = 3, Ls =
+// 32: 8% off); there the scan runs the other way in 1/a (K_INVR): with Q_s =
+// sum_{t>=s} a^(s-t) x_t,
+//   w_s = a^(s-Ls) / (a^-Ls + mf) Q_0 - Q_(s+1) / a.
 //
 // The four passes of M_pc^+ M_pc at 32^4 x 16 in FP32 (L_B, L_POST, two
 // L_BMINV: 9 fields, 7.2 GB, 1.07 ms at the measured peak) take 1.07 ms; with
 // one element per thread staged in shared memory, and the inverse as a dense
 // Ls x Ls product, they took 1.47 ms (BF16 at 24^4 x 16: 0.48 -> 0.29 ms).
 #include <algorithm>
+#include <cmath>
 
 #include "dev_common.cuh"
 #include "dwf_internal.cuh"
@@ -46,7 +51,8 @@ struct LocalArgs {
     float c0, c1;                // out = scale (c0 x + c1 S x) (the inverse: of w, scale folded in)
     float z0, z1;                // L_POST: out = c0 x + c1 S x + scale (z0 z + z1 S z)
     float mf;
-    float a, wall;               // inverse: a, mf / (1 + mf a^Ls)
+    float a, wall;               // inverse: a, mf / (1 + mf a^Ls) (K_INVR: 1/a)
+    double a64, kappa;           // K_INVR: 1/a, 1 / (a^-Ls + mf)
     float* cg_x;
     float* cg_r;
     float* cg_p;
@@ -58,7 +64,7 @@ struct LocalArgs {
     float lin_a, lin_bu, lin_bv;
 };
 
-enum { K_ONE = 0, K_POST = 1, K_PB = 2, K_INV = 3 };
+enum { K_ONE = 0, K_POST = 1, K_PB = 2, K_INV = 3, K_INVR = 4 };
 constexpr int kLocalThreads = 256;
 
 // Where a thread's row continues: the threads holding the next lane down and
@@ -84,7 +90,8 @@ __device__ __forceinline__ void shift_sum(float c0, float c1, const float (&x)[V
 
 template <class Sin, class Sin2, class Sout, int VL, int KIND>
 __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
-    constexpr int kU = KIND == K_ONE || KIND == K_INV ? 4 : 2;
+    constexpr bool INV = KIND == K_INV || KIND == K_INVR, REV = KIND == K_INVR;
+    constexpr int kU = KIND == K_ONE || INV ? 4 : 2;
     __shared__ double s_red[kLocalThreads];
     const int Ls = a.Ls, nrhs = a.nrhs, TPR = Ls / VL;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -99,7 +106,18 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
     rp.f_up = pos < TPR - 1 ? 1.f : -a.mf;
     // inverse: powers of a for the scan
     float pw[VL], astep = 1.f, base_dn = 1.f, base_up = 1.f;
-    if (KIND == K_INV) {
+    double astep64 = 1.0;
+    if (REV) {   // powers in FP64: |a| near 1 keeps their rounding, and kappa alone may be beyond FP32
+        double q = 1.0, dn = a.kappa, up = a.kappa;
+#pragma unroll
+        for (int v = 0; v < VL; ++v) { pw[v] = (float)q; q *= a.a64; }
+        astep64 = q;
+        astep = (float)q;
+        for (int i = 0; i < s0 + 1; ++i) dn *= a.a64;
+        for (int i = 0; i < Ls - s0 - VL + 1; ++i) up *= a.a64;
+        base_dn = (float)dn;
+        base_up = (float)up;
+    } else if (INV) {
         float q = 1.f;
 #pragma unroll
         for (int v = 0; v < VL; ++v) { pw[v] = q; q *= a.a; }   // a^v
@@ -156,15 +174,16 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
                 }
                 if (ok && live) store_lanes<float, VL, float>(a.cg_p + 2 * g, xr[u], xi[u]);
             }
-            if (KIND == K_INV) {
-                // mirrored lanes for S_+: m runs with the recurrence
-                const int j = down ? pos : TPR - 1 - pos;
-                const int step = down ? 1 : -1;
+            if (INV) {
+                // mirrored lanes for S_+ (K_INVR: for S_-): m runs with the recurrence
+                const bool fwd = down != REV;
+                const int j = fwd ? pos : TPR - 1 - pos;
+                const int step = fwd ? 1 : -1;
                 float wr[VL], wi[VL];
 #pragma unroll
                 for (int v = 0; v < VL; ++v) {
-                    wr[v] = down ? xr[u][v] : xr[u][VL - 1 - v];
-                    wi[v] = down ? xi[u][v] : xi[u][VL - 1 - v];
+                    wr[v] = fwd ? xr[u][v] : xr[u][VL - 1 - v];
+                    wi[v] = fwd ? xi[u][v] : xi[u][VL - 1 - v];
                 }
 #pragma unroll
                 for (int v = 1; v < VL; ++v) {
@@ -173,16 +192,26 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
                 }
                 // inclusive scan of the thread totals, then the carry from the thread before
                 float totr = wr[VL - 1], toti = wi[VL - 1], f = astep;
-                for (int o = 1; o < TPR; o <<= 1, f *= f) {
+                double f64 = astep64;
+                for (int o = 1; o < TPR; o <<= 1) {
                     const float br = __shfl_sync(0xffffffffu, totr, j >= o ? lane - step * o : lane);
                     const float bi = __shfl_sync(0xffffffffu, toti, j >= o ? lane - step * o : lane);
                     if (j >= o) { totr = fmaf(f, br, totr); toti = fmaf(f, bi, toti); }
+                    if (REV) { f64 *= f64; f = (float)f64; }
+                    else f *= f;
                 }
                 const int prev = j > 0 ? lane - step : lane, last = lane + step * (TPR - 1 - j);
                 const float cr = __shfl_sync(0xffffffffu, totr, prev), ci = __shfl_sync(0xffffffffu, toti, prev);
                 const float lr = __shfl_sync(0xffffffffu, totr, last), li = __shfl_sync(0xffffffffu, toti, last);
-                const float wall = -a.wall * (down ? base_dn : base_up);
-                const float carry = j > 0 ? a.a : 0.f;
+                const float base = fwd ? base_dn : base_up;
+                const float wall = REV ? base : -a.wall * base;
+                float carry = j > 0 ? a.a : 0.f;
+                if (REV) {   // -Q of the next lane in the recurrence's order, over a
+                    carry = -carry;
+#pragma unroll
+                    for (int v = VL - 1; v > 0; --v) { wr[v] = -a.a * wr[v - 1]; wi[v] = -a.a * wi[v - 1]; }
+                    wr[0] = wi[0] = 0.f;
+                }
 #pragma unroll
                 for (int v = 0; v < VL; ++v) {
                     wr[v] = fmaf(pw[v], fmaf(wall, lr, carry * cr), wr[v]);
@@ -190,11 +219,11 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
                 }
 #pragma unroll
                 for (int v = 0; v < VL; ++v) {
-                    xr[u][v] = down ? wr[v] : wr[VL - 1 - v];
-                    xi[u][v] = down ? wi[v] : wi[VL - 1 - v];
+                    xr[u][v] = fwd ? wr[v] : wr[VL - 1 - v];
+                    xi[u][v] = fwd ? wi[v] : wi[VL - 1 - v];
                 }
             }
-            if (KIND == K_INV && a.c1 == 0.f) {
+            if (INV && a.c1 == 0.f) {
 #pragma unroll
                 for (int v = 0; v < VL; ++v) { yr[v] = a.c0 * xr[u][v]; yi[v] = a.c0 * xi[u][v]; }
             } else {
@@ -291,13 +320,17 @@ static dwf_status launch_vl(dwf_handle* h, const LocalCall& c, const TileSet& ts
     switch (c.op) {
         case L_MINV:
         case L_BMINV: {
-            double aL = 1.0;
-            for (int i = 0; i < f.Ls; ++i) aL *= f.a;
-            a.a = (float)f.a;
-            a.wall = (float)(f.mf / (1.0 + f.mf * aL));
+            const bool rev = std::abs(f.a) > 1.0;
+            const double r = rev ? 1.0 / f.a : f.a;
+            double rL = 1.0;
+            for (int i = 0; i < f.Ls; ++i) rL *= r;
+            a.a = (float)r;
+            a.a64 = r;
+            if (rev) a.kappa = 1.0 / (rL + f.mf);
+            else a.wall = (float)(f.mf / (1.0 + f.mf * rL));
             a.c0 = (float)(c.scale * f.inv_d * (c.op == L_BMINV ? f.b5 : 1.0));
             a.c1 = (float)(c.op == L_BMINV ? c.scale * f.inv_d * f.c5 : 0.0);
-            kern = k_local<Sin, Sin2, Sout, VL, K_INV>;
+            kern = rev ? k_local<Sin, Sin2, Sout, VL, K_INVR> : k_local<Sin, Sin2, Sout, VL, K_INV>;
             break;
         }
         case L_POST:
