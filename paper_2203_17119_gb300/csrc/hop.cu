@@ -17,6 +17,7 @@
 //            MOO     out = M_oo x + scale * Dh in  (+ per-tile |out|^2),
 //            the last step of the Schur operator M_pc = M_oo - M_oe M_ee^-1 M_eo.
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <type_traits>
 #include <map>
@@ -1446,6 +1447,7 @@ bool hop_post_ok(const dwf_handle* h, dwf_prec op, dwf_prec vec, int nrhs, int V
 
 bool hop_bminv_ok(const dwf_handle* h, dwf_prec op, int nrhs, int VL) {
     if (op != DWF_FP32 && op != DWF_BF16) return false;
+    if (std::abs(h->f5[0].a) > 1.0) return false;   // the epilogue's scan grows like |a|^Ls
     const int n5 = h->p.Ls * nrhs;
     const int vl = op == DWF_BF16 ? 2 : (VL == 1 ? 1 : 2);
     const int tps = n5 / vl;

@@ -20,10 +20,14 @@
 // obeys w_s = x_s + a w_{s-1} (S_-; S_+ the mirror image) and
 //   w_0 = [x_0 - mf sum_{t>=1} a^(Ls-t) x_t] / (1 + mf a^Ls),
 // one multiply-add per element for the sum, one for the recurrence, and the
-// output is c w_s or c0 w_s + c1 w_{s-1} with 1/d and the scale folded in.  A
-// thread takes the real or the imaginary part of one row; rows lie in shared
+// output is c w_s or c0 w_s + c1 w_{s-1} with 1/d and the scale folded in.
+// For |a| > 1 (c5 well above b5) that recurrence loses a factor |a|^Ls; it runs
+// the other way there (REV), from
+//   w_{Ls-1} = sum_t a^-t x_t / (a (a^-Ls + mf)),  w_{s-1} = (w_s - x_s) / a.
+// A thread takes the real or the imaginary part of one row; rows lie in shared
 // memory Ls + 1 complex numbers apart (Ls is even: no bank conflicts).
 #include <algorithm>
+#include <cmath>
 
 #include "dev_common.cuh"
 #include "dwf_internal.cuh"
@@ -155,13 +159,13 @@ struct Minv64Args {
     double2* out;
     const int4* tiles;
     int Ls, nrhs, dagger;
-    double a, mf, wall;   // wall = 1 / (1 + mf a^Ls)
+    double a, mf, wall;   // wall = 1 / (1 + mf a^Ls); REV: a is 1/a, wall = a / (a^Ls + mf) with that a
     double c0, c1;        // out = c0 w_s + c1 w_{s -+ 1}
 };
 
 constexpr int kM64Rows = 64;
 
-template <bool B>
+template <bool B, bool REV>
 __global__ void __launch_bounds__(2 * kM64Rows) k_minv64(const Minv64Args a) {
     extern __shared__ __align__(16) double2 sm64[];
     const int Ls = a.Ls, nrhs = a.nrhs, stride = Ls + 1, tid = threadIdx.x;
@@ -182,17 +186,31 @@ __global__ void __launch_bounds__(2 * kM64Rows) k_minv64(const Minv64Args a) {
             // S_-: first = 0, upwards; S_+: first = Ls - 1, downwards
             const int first = down ? 0 : 2 * (Ls - 1), st = down ? 2 : -2;
             double acc = 0.0;
-            for (int k = 1; k < Ls; ++k) acc = fma(acc, a.a, part[first + k * st]);
-            const double w0 = fma(-a.mf * a.a, acc, part[first]) * a.wall;
-            double w = w0;
-            for (int k = 1; k < Ls; ++k) {
-                const int i = first + k * st;
-                const double wn = fma(a.a, w, part[i]);
-                part[i] = B ? fma(a.c1, w, a.c0 * wn) : a.c0 * wn;
-                w = wn;
+            if (REV) {
+                const int last = first + (Ls - 1) * st;
+                for (int k = 0; k < Ls; ++k) acc = fma(acc, a.a, part[last - k * st]);
+                const double top = a.wall * acc;
+                double w = top;
+                for (int k = 0; k < Ls - 1; ++k) {
+                    const int i = last - k * st;
+                    const double wn = a.a * (w - part[i]);
+                    part[i] = B ? fma(a.c1, wn, a.c0 * w) : a.c0 * w;
+                    w = wn;
+                }
+                part[first] = B ? fma(a.c1 * -a.mf, top, a.c0 * w) : a.c0 * w;
+            } else {
+                for (int k = 1; k < Ls; ++k) acc = fma(acc, a.a, part[first + k * st]);
+                const double w0 = fma(-a.mf * a.a, acc, part[first]) * a.wall;
+                double w = w0;
+                for (int k = 1; k < Ls; ++k) {
+                    const int i = first + k * st;
+                    const double wn = fma(a.a, w, part[i]);
+                    part[i] = B ? fma(a.c1, w, a.c0 * wn) : a.c0 * wn;
+                    w = wn;
+                }
+                // S w at the first lane: -mf times the last one
+                part[first] = B ? fma(a.c1 * -a.mf, w, a.c0 * w0) : a.c0 * w0;
             }
-            // S w at the first lane: -mf times the last one
-            part[first] = B ? fma(a.c1 * -a.mf, w, a.c0 * w0) : a.c0 * w0;
         }
         __syncthreads();
         double2* out = a.out + base + (int64_t)rb * Ls;
@@ -213,9 +231,16 @@ dwf_status launch_local64(dwf_handle* h, const LocalCall& c, const TileSet& ts, 
         a.Ls = Ls;
         a.nrhs = c.nrhs;
         a.dagger = c.dagger;
+        const bool rev = std::abs(f.a) > 1.0;
         a.a = f.a;
         a.mf = f.mf;
         a.wall = f.inv_den * f.d;
+        if (rev) {
+            a.a = 1.0 / f.a;
+            double rL = 1.0;
+            for (int i = 0; i < Ls; ++i) rL *= a.a;
+            a.wall = a.a / (rL + f.mf);
+        }
         a.c0 = c.scale * f.inv_d * (c.op == L_BMINV ? f.b5 : 1.0);
         a.c1 = c.op == L_BMINV ? c.scale * f.inv_d * f.c5 : 0.0;
         if (c.partial != nullptr || c.out == nullptr || c.cg_r != nullptr) {
@@ -223,8 +248,9 @@ dwf_status launch_local64(dwf_handle* h, const LocalCall& c, const TileSet& ts, 
             return DWF_ERR_UNSUPPORTED;
         }
         const size_t smem = (size_t)kM64Rows * (Ls + 1) * sizeof(double2);
-        if (c.op == L_BMINV) k_minv64<true><<<nt, 2 * kM64Rows, smem, s>>>(a);
-        else k_minv64<false><<<nt, 2 * kM64Rows, smem, s>>>(a);
+        void (*kern)(const Minv64Args) = c.op == L_BMINV ? (rev ? k_minv64<true, true> : k_minv64<true, false>)
+                                                         : (rev ? k_minv64<false, true> : k_minv64<false, false>);
+        kern<<<nt, 2 * kM64Rows, smem, s>>>(a);
     } else {
         Local64Args a{};
         a.in = (const double2*)c.in;

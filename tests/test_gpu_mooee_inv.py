@@ -69,3 +69,29 @@ def test_schur_operator(Ls, dagger, prec):
     h.mpc(out, src, dagger, prec)
     got = LY.from_cb(_host(out), DIMS, None, 1, Ls)[0][0]
     assert LY.rel_l2(got, O.mpc(U, vals[0], prm, dagger)) <= TOL_MPC[prec]
+
+
+@pytest.mark.parametrize("dagger", [False, True])
+@pytest.mark.parametrize("Ls,nrhs", [(2, 1), (10, 2), (24, 1), (32, 2)])
+@pytest.mark.parametrize("b5,c5,mf", ACTIONS)
+def test_inverse_fp64(b5, c5, mf, Ls, nrhs, dagger):
+    U, h, psi, prm = _setup(Ls, b5, c5, mf, nrhs)
+    src, vals = _dev(psi, G.FP64)
+    out = torch.empty_like(src)
+    h.mooee_inv(out, src, 1, dagger, G.FP64, nrhs)
+    got = LY.from_cb(_host(out), DIMS, None, 1, Ls)[0]
+    for g, v in zip(got, vals):   # sums of up to 32 terms, a few roundings of 2^-53 each, on both sides
+        assert LY.rel_l2(g, O.mooee_inv(v, prm, dagger)) <= 128 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("prec", [G.FP32, G.BF16])
+@pytest.mark.parametrize("dagger", [False, True])
+@pytest.mark.parametrize("Ls", [16, 32])
+def test_schur_operator_with_fusion_chosen(Ls, dagger, prec):
+    U, h, psi, prm = _setup(Ls, 0.5, 2.5, 0.01)
+    h.set_fusion(1, True)
+    src, vals = _dev(psi, prec)
+    out = torch.empty_like(src)
+    h.mpc(out, src, dagger, prec)
+    got = LY.from_cb(_host(out), DIMS, None, 1, Ls)[0][0]
+    assert LY.rel_l2(got, O.mpc(U, vals[0], prm, dagger)) <= TOL_MPC[prec]
