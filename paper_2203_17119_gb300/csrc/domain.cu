@@ -238,13 +238,14 @@ __global__ void k_gather_links(const double* __restrict__ U, const int64_t* __re
 
 // Range of the links' sizes: the biased exponents of the largest element of
 // any link, and of the smallest link's largest element (links of zeros aside);
-// a NaN or infinity has exponent 2047.
+// an element up to 1.125 2^k counts as below 2^k (unit links, and 1 + rounding,
+// then take the unit of the links within them); a NaN or infinity has exponent 2046 or 2047.
 __global__ void k_link_range(const double* __restrict__ l64, int64_t n /* sites * 8 */, int* __restrict__ range) {
     int hi = 0, lo = 4096;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         int e = 0;
 #pragma unroll
-        for (int j = 0; j < 18; ++j) e = max(e, (__double2hiint(l64[i * 18 + j]) >> 20) & 0x7ff);
+        for (int j = 0; j < 18; ++j) e = max(e, ((__double2hiint(l64[i * 18 + j]) & 0x7fffffff) - 0x20000) >> 20);
         if (e > 0) {
             hi = max(hi, e);
             lo = min(lo, e);
@@ -259,7 +260,7 @@ __global__ void k_link_range(const double* __restrict__ l64, int64_t n /* sites 
 }
 
 // Fixed-point links: w = (hi 2^32 + lo) 2^(exp - 61), lo a signed word above
-// -2^31, with |w| < 2^exp.  Covered (info[1] = 1): finite links whose sizes differ by at
+// -2^31, with |w| < 1.125 2^exp.  Covered (info[1] = 1): finite links whose sizes differ by at
 // most 2^8, so that the common unit costs none of them precision against FP64
 // (SU(3) links lie within a factor sqrt(3)), of a size that leaves the
 // result's exponent in range.

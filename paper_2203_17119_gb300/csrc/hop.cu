@@ -374,26 +374,40 @@ __device__ __forceinline__ void hop_dir(const Sin* __restrict__ in, const int* s
 // GB300 has 2 FP64 lanes per clock and SM against 32 for the 32 x 32 -> 64-bit
 // integer multiply-add, and the hop's 1320 flops per lane are what bounds the
 // FP64 form (91% of the FP64 pipe).  So the FP64 hop transports in 64-bit
-// fixed point: links as w = (w1 2^32 + w0) 2^(exp - 61), |w1| <= 2^29, w0 a
-// signed word (set_gauge); the projected half spinors h as integers in units
+// fixed point: links as w = (w1 2^32 + w0) 2^(exp - 61), |w| < 1.125 2^exp, w0
+// a signed word (set_gauge); the projected half spinors h as integers in units
 // of 2^(E - 1080), E one above the largest biased exponent of any component
-// met so far for this site and lane -- so |h| < 2^59 units, and when a larger
+// met so far for this site and lane -- so |h| < 2^58 units, and when a larger
 // one arrives the accumulators are shifted to the new unit.  With h = h1 2^32
 // + h0 a real product is three multiply-adds,
 //   w h 2^-64 = w1 h1 + (w1 h0 + w0 h1) 2^-32 + O(2^-2),
 // the second sum enters the first by its high word (rounded: it starts at
 // 2^31), and the colour sum and the sum over directions are integer adds.
-// Bounds: the two product sums stay below 6 2^56 and 6 (2^60 + 2^58) < 2^63,
-// the sum over directions below 2^62, for any |w| <= 1.  A result is within a
-// few of its units, 2^-52 of a component's rms, before one rounding to FP64;
-// FP64 arithmetic rounds every operation by 2^-53, and the error against exact
-// arithmetic comes out no larger than the FP64 form's.  Lanes the fixed point
-// does not cover -- a NaN, an infinity, all components below 2^-895 or one
-// above 2^56 -- run the FP64 form; so does a handle whose links differ in size
-// by more than 2^8 (set_gauge).  Measured, bare hop: 16^4 x 12 650 -> 209 us,
-// 24^4 x 16 4.17 -> 1.34 ms (FP64 form -> this); no pipe is full (FP64 half,
-// integer multiply-add about 60%): the chains of dependent integer
-// instructions at 16 warps per SM are what is left.
+// Bounds: the two product sums stay below 6 1.125 2^55 and 6 (1.125 2^60 +
+// 2^57) < 2^63, the sum over directions below 2^62.
+//
+// Every number keeps FP64's precision, not only the largest.  A result is off
+// by at most 25 of its units u (2.8 a direction: 2^-2 for each of six dropped
+// w0 h0, 1/2 for the rounded high word, the rest for w and h; 2 for changes of
+// the unit), about one u rms; the FP64 form by up to 16 2^-53 of the sum of
+// the moduli of its terms.  So a lane keeps the fixed-point sums only where
+// the terms of every one of its numbers reach 1.25 2^52 u: M adds, over the
+// directions, the smallest |g| (larger of its parts) of the transported half
+// spinor, and each number takes one g from every direction.  On Gaussian
+// fields one lane in 10^5 fails that (the median of M is 2^54.3 u) and the
+// error is 0.58 of the FP64 form's; where a third of the lanes are just
+// covered it comes to about twice the FP64 form's (rms).  Lanes that fail run
+// the FP64 form -- numbers that a larger one does not reach: links that do not
+// mix two colours, a neighbour that the projector annihilates, one neighbour
+// far above the others --, and so do a NaN, an infinity, all components below
+// 2^-895 or one above 2^56, and a handle whose links differ in size by more
+// than 2^8 (set_gauge).  Telling them costs 2.4% (D in FP64 at 24^4 x 16 4.46
+// -> 4.57 ms).
+//
+// Measured, bare hop: 16^4 x 12 650 -> 209 us, 24^4 x 16 4.17 -> 1.34 ms (FP64
+// form -> this); no pipe is full (FP64 half, integer multiply-add about 60%):
+// the chains of dependent integer instructions at 16 warps per SM are what is
+// left.
 //
 // Half of the projections and conversions (spin 0) run on the FP64 pipe (an
 // add, an exponent add, a conversion), half (spin 1) as shifts of the
@@ -402,6 +416,7 @@ __device__ __forceinline__ void hop_dir(const Sin* __restrict__ in, const int* s
 struct FxLink {
     int hi, lo;
 };
+constexpr int kFxCover = 0x140000;   // 1.25 2^52, high word
 
 // |x| of the double v: mantissa aligned to bit 63, moved down by E + 6 - e;
 // EB = (E + 6) << 21 | 0x1fffff
@@ -533,16 +548,21 @@ __device__ __forceinline__ void fx_row(const int4 (&v)[3], const FxHalf& h, long
     }
 }
 
+// high word of the larger part of g
+__device__ __forceinline__ int fx_size(long long r, long long i) {
+    return max(abs((int)(r >> 32)), abs((int)(i >> 32)));
+}
+
 // Direction +mu (k < 4) or -mu in fixed point: acc += W h on the upper spins,
-// rebuilt lower spins; E the accumulators' unit, bad set where the FP64 form
-// has to decide (denormals only).
+// rebuilt lower spins; E the accumulators' unit, M the sum of the smallest |g|
+// (high words), bad set where the FP64 form has to decide (denormals only).
 template <int MU, bool DAG>
 __device__ __forceinline__ void hop_dir_fx(int k, const double* __restrict__ in, const int* s_nbr,
                                            const FxLink* s_link, int N5, int lane0, long long (&ar)[12],
-                                           long long (&ai)[12], int& E, bool& bad) {
+                                           long long (&ai)[12], int& E, int& M, bool& bad) {
     const int nb = s_nbr[k];
     if (nb < 0) return;
-    const int P = ((k < 4) != DAG) ? 0 : -1, M = ~P;   // SG = +1 for (1 - g_mu)
+    const int P = ((k < 4) != DAG) ? 0 : -1, Pm = ~P;   // SG = +1 for (1 - g_mu)
     const double2* src = reinterpret_cast<const double2*>(in) + ((int64_t)nb * 12 * N5 + lane0);
     double2 x[12];
 #pragma unroll
@@ -555,17 +575,20 @@ __device__ __forceinline__ void hop_dir_fx(int k, const double* __restrict__ in,
         if (E > 0) {
 #pragma unroll
             for (int c = 0; c < 12; ++c) { ar[c] >>= d; ai[c] >>= d; }
+            M >>= min(d, 31);
         }
         E = Ed + 1;
     }
     FxHalf h;
     fx_project<MU>(x, P, E, h);
     const int4* w = reinterpret_cast<const int4*>(s_link) + k * 9;
+    int least = 0x7fffffff;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const int4 v[3] = {w[a * 3], w[a * 3 + 1], w[a * 3 + 2]};
         long long gr[2], gi[2];
         fx_row(v, h, gr, gi);
+        least = min(least, min(fx_size(gr[0], gi[0]), fx_size(gr[1], gi[1])));
         // rebuild: upper += g, lower += -SG A_mu^+ g
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -574,14 +597,15 @@ __device__ __forceinline__ void hop_dir_fx(int k, const double* __restrict__ in,
             ar[q * 3 + a] += gr[q];
             ai[q * 3 + a] += gi[q];
             if (fx_itype(MU)) {
-                fx_add(ar[low], gi[q], plus ? M : P);
-                fx_add(ai[low], gr[q], plus ? P : M);
+                fx_add(ar[low], gi[q], plus ? Pm : P);
+                fx_add(ai[low], gr[q], plus ? P : Pm);
             } else {
-                fx_add(ar[low], gr[q], plus ? P : M);
-                fx_add(ai[low], gi[q], plus ? P : M);
+                fx_add(ar[low], gr[q], plus ? P : Pm);
+                fx_add(ai[low], gi[q], plus ? P : Pm);
             }
         }
     }
+    M += least;
 }
 
 // The FP64 form of one site and lane (out of line: rarely taken)
@@ -611,18 +635,18 @@ __device__ __forceinline__ double hop_site_fx(const double* __restrict__ in, con
     long long r[12], i[12];
 #pragma unroll
     for (int c = 0; c < 12; ++c) r[c] = i[c] = 0;
-    int E = 0;
+    int E = 0, M = 0;
     bool bad = false;
 #pragma unroll 1
-    for (int k = 0; k < 8; k += 4) hop_dir_fx<0, DAG>(k, in, nb, lk, N5, lane0, r, i, E, bad);
+    for (int k = 0; k < 8; k += 4) hop_dir_fx<0, DAG>(k, in, nb, lk, N5, lane0, r, i, E, M, bad);
 #pragma unroll 1
-    for (int k = 1; k < 8; k += 4) hop_dir_fx<1, DAG>(k, in, nb, lk, N5, lane0, r, i, E, bad);
+    for (int k = 1; k < 8; k += 4) hop_dir_fx<1, DAG>(k, in, nb, lk, N5, lane0, r, i, E, M, bad);
 #pragma unroll 1
-    for (int k = 2; k < 8; k += 4) hop_dir_fx<2, DAG>(k, in, nb, lk, N5, lane0, r, i, E, bad);
+    for (int k = 2; k < 8; k += 4) hop_dir_fx<2, DAG>(k, in, nb, lk, N5, lane0, r, i, E, M, bad);
 #pragma unroll 1
-    for (int k = 3; k < 8; k += 4) hop_dir_fx<3, DAG>(k, in, nb, lk, N5, lane0, r, i, E, bad);
+    for (int k = 3; k < 8; k += 4) hop_dir_fx<3, DAG>(k, in, nb, lk, N5, lane0, r, i, E, M, bad);
     // E = 0: every neighbour component is zero (or the FP64 form runs)
-    if (((E != 0 || bad) && (E < 128 || E > 1080)) || info.y == 0) {
+    if (((E != 0 || bad) && (E < 128 || E > 1080 || M < kFxCover)) || info.y == 0) {
         double tr[12], ti[12];
         hop_fx_fallback<DAG>(in, nb, lk64, N5, lane0, tr, ti);
 #pragma unroll
@@ -1145,16 +1169,11 @@ __global__ void __launch_bounds__(256, 2) k_hop_fx_split(const HopArgs a) {
                 bad |= s_E[d][j] < 0;
             }
             double re[2], im[2], factor;
-            if (((Em != 0 || bad) && (Em < 128 || Em > 1080)) || info.y == 0) {
-                double tr[12], ti[12];
-                hop_fx_fallback<DAG>(in, a.nbr + site * 8, a.links64 + site * 144, N5, lane0, tr, ti);
-#pragma unroll
-                for (int c = 0; c < 12; ++c)
-                    if (c >> 1 == k) { re[c & 1] = tr[c]; im[c & 1] = ti[c]; }
-                factor = 1.0;
-            } else {
+            bool fp64 = ((Em != 0 || bad) && (Em < 128 || Em > 1080)) || info.y == 0;
+            if (!fp64) {
                 const bool upper = k < 3;   // rows 2 k, 2 k + 1: upper spins for k < 3
                 long long sr[2] = {0, 0}, si[2] = {0, 0};
+                int size[2] = {0, 0};       // each row's own sum of |g| decides here
 #pragma unroll
                 for (int d = 0; d < 8; ++d) {
                     const int Ek = s_E[d][j];
@@ -1166,6 +1185,7 @@ __global__ void __launch_bounds__(256, 2) k_hop_fx_split(const HopArgs a) {
                         const int c = 2 * k + e, spin = c / 3, col = c - 3 * spin;
                         const int q = upper ? spin : (mu < 2 ? 3 - spin : spin - 2);
                         const long long gr = s_g[d][(q * 3 + col) * 2][j] >> dn, gi = s_g[d][(q * 3 + col) * 2 + 1][j] >> dn;
+                        size[e] += fx_size(gr, gi);
                         if (upper) {
                             sr[e] += gr;
                             si[e] += gi;
@@ -1179,6 +1199,15 @@ __global__ void __launch_bounds__(256, 2) k_hop_fx_split(const HopArgs a) {
 #pragma unroll
                 for (int e = 0; e < 2; ++e) { re[e] = __ll2double_rn(sr[e]); im[e] = __ll2double_rn(si[e]); }
                 factor = __hiloint2double(max(Em + info.x - 54, 1) << 20, 0);
+                fp64 = Em != 0 && min(size[0], size[1]) < kFxCover;
+            }
+            if (fp64) {
+                double tr[12], ti[12];
+                hop_fx_fallback<DAG>(in, a.nbr + site * 8, a.links64 + site * 144, N5, lane0, tr, ti);
+#pragma unroll
+                for (int c = 0; c < 12; ++c)
+                    if (c >> 1 == k) { re[c & 1] = tr[c]; im[c & 1] = ti[c]; }
+                factor = 1.0;
             }
             const double sc = a.scale * factor;
             const int s = lane0 % Ls;
