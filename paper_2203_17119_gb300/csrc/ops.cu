@@ -29,6 +29,16 @@ int tile_for(dwf_handle* h, int nrhs) {
     return h->default_T;
 }
 
+// Numbers of ordinary size, -1 <= x < 1, for the FP64 hop to be timed on: its
+// fixed-point form leaves out the work for a neighbour that is all zero.
+__global__ void k_tune_fill(double* __restrict__ x, int64_t n) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        uint32_t v = (uint32_t)i * 2654435761u;
+        v = (v ^ (v >> 15)) * 2246822519u;
+        x[i] = (double)(int)(v ^ (v >> 13)) * 0x1p-31;
+    }
+}
+
 // Autotuner: for each candidate (tile size, lanes per thread) time what a
 // CG iteration applies, M_pc and M_pc^+ with the operator of precision
 // `prec` (the hops and the fifth-dimension kernels share the tile table; for
@@ -44,7 +54,13 @@ dwf_status autotune(dwf_handle* h, int nrhs, dwf_prec prec, int* best) {
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     const size_t bytes = cb_elems(h, 1, nrhs) * 2 * prec_size(prec);
-    cudaMemsetAsync(h->d_tmp2, 0, bytes, s);
+    if (prec == DWF_FP64) {
+        k_tune_fill<<<152 * 8, 256, 0, s>>>((double*)h->d_tmp2, (int64_t)(bytes / sizeof(double)));
+        note_launch();
+        DWF_CUDA(cudaGetLastError());
+    } else {
+        cudaMemsetAsync(h->d_tmp2, 0, bytes, s);
+    }
     // FP32 / BF16 fields: two per FP64-sized scratch field
     unsigned char* t1 = reinterpret_cast<unsigned char*>(h->d_tmp);
     unsigned char* t2 = reinterpret_cast<unsigned char*>(h->d_tmp2);
