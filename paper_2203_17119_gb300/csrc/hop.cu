@@ -391,20 +391,23 @@ __device__ __forceinline__ void hop_dir(const Sin* __restrict__ in, const int* s
 // w0 h0, 1/2 for the rounded high word, the rest for w and h; 2 for changes of
 // the unit), about one u rms; the FP64 form by up to 16 2^-53 of the sum of
 // the moduli of its terms.  So a lane keeps the fixed-point sums only where
-// the terms of every one of its numbers reach 1.25 2^52 u: M adds, over the
-// directions, the smallest |g| (larger of its parts) of the transported half
-// spinor, and each number takes one g from every direction.  On Gaussian
-// fields one lane in 10^5 fails that (the median of M is 2^54.3 u) and the
-// error is 0.58 of the FP64 form's; where a third of the lanes are just
+// the terms of every one of its numbers reach 1.25 2^52 u: M adds, colour by
+// colour and over the directions, the smaller |g| (larger of its parts) of the
+// two transported spins, and each number takes one g from every direction.
+// None of 2.4 M Gaussian lanes failed that (the median of M is 2^54.9 u, their
+// least 2^52.6), and the error is 0.58 of the FP64 form's; where a third of the lanes are just
 // covered it comes to about twice the FP64 form's (rms).  Lanes that fail run
 // the FP64 form -- numbers that a larger one does not reach: links that do not
 // mix two colours, a neighbour that the projector annihilates, one neighbour
 // far above the others --, and so do a NaN, an infinity, all components below
 // 2^-895 or one above 2^56, and a handle whose links differ in size by more
-// than 2^8 (set_gauge).  Telling them costs 2.4% (D in FP64 at 24^4 x 16 4.46
-// -> 4.57 ms).
+// than 2^8 (set_gauge).  A warp with one such lane takes some 25 us longer, a
+// fixed tail on small lattices: with the smallest |g| of all six components in
+// one sum, one Gaussian lane in 10^5 failed, and 16^4 x 12 took 233 to 245 us
+// instead of 217.  Telling them costs 3% of the bare hop (16^4 x 12 209 -> 217
+// us).
 //
-// Measured, bare hop: 16^4 x 12 650 -> 209 us, 24^4 x 16 4.17 -> 1.34 ms (FP64
+// Measured, bare hop: 16^4 x 12 650 -> 217 us, 24^4 x 16 4.17 -> 1.37 ms (FP64
 // form -> this); no pipe is full (FP64 half, integer multiply-add about 60%):
 // the chains of dependent integer instructions at 16 warps per SM are what is
 // left.
@@ -554,12 +557,12 @@ __device__ __forceinline__ int fx_size(long long r, long long i) {
 }
 
 // Direction +mu (k < 4) or -mu in fixed point: acc += W h on the upper spins,
-// rebuilt lower spins; E the accumulators' unit, M the sum of the smallest |g|
-// (high words), bad set where the FP64 form has to decide (denormals only).
+// rebuilt lower spins; E the accumulators' unit, M per colour the sum of the
+// smaller |g| (high words), bad set where the FP64 form has to decide (denormals only).
 template <int MU, bool DAG>
 __device__ __forceinline__ void hop_dir_fx(int k, const double* __restrict__ in, const int* s_nbr,
                                            const FxLink* s_link, int N5, int lane0, long long (&ar)[12],
-                                           long long (&ai)[12], int& E, int& M, bool& bad) {
+                                           long long (&ai)[12], int& E, int (&M)[3], bool& bad) {
     const int nb = s_nbr[k];
     if (nb < 0) return;
     const int P = ((k < 4) != DAG) ? 0 : -1, Pm = ~P;   // SG = +1 for (1 - g_mu)
@@ -575,20 +578,20 @@ __device__ __forceinline__ void hop_dir_fx(int k, const double* __restrict__ in,
         if (E > 0) {
 #pragma unroll
             for (int c = 0; c < 12; ++c) { ar[c] >>= d; ai[c] >>= d; }
-            M >>= min(d, 31);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) M[c] >>= min(d, 31);
         }
         E = Ed + 1;
     }
     FxHalf h;
     fx_project<MU>(x, P, E, h);
     const int4* w = reinterpret_cast<const int4*>(s_link) + k * 9;
-    int least = 0x7fffffff;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const int4 v[3] = {w[a * 3], w[a * 3 + 1], w[a * 3 + 2]};
         long long gr[2], gi[2];
         fx_row(v, h, gr, gi);
-        least = min(least, min(fx_size(gr[0], gi[0]), fx_size(gr[1], gi[1])));
+        M[a] += min(fx_size(gr[0], gi[0]), fx_size(gr[1], gi[1]));
         // rebuild: upper += g, lower += -SG A_mu^+ g
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -605,7 +608,6 @@ __device__ __forceinline__ void hop_dir_fx(int k, const double* __restrict__ in,
             }
         }
     }
-    M += least;
 }
 
 // The FP64 form of one site and lane (out of line: rarely taken)
@@ -635,7 +637,7 @@ __device__ __forceinline__ double hop_site_fx(const double* __restrict__ in, con
     long long r[12], i[12];
 #pragma unroll
     for (int c = 0; c < 12; ++c) r[c] = i[c] = 0;
-    int E = 0, M = 0;
+    int E = 0, M[3] = {0, 0, 0};
     bool bad = false;
 #pragma unroll 1
     for (int k = 0; k < 8; k += 4) hop_dir_fx<0, DAG>(k, in, nb, lk, N5, lane0, r, i, E, M, bad);
@@ -646,7 +648,7 @@ __device__ __forceinline__ double hop_site_fx(const double* __restrict__ in, con
 #pragma unroll 1
     for (int k = 3; k < 8; k += 4) hop_dir_fx<3, DAG>(k, in, nb, lk, N5, lane0, r, i, E, M, bad);
     // E = 0: every neighbour component is zero (or the FP64 form runs)
-    if (((E != 0 || bad) && (E < 128 || E > 1080 || M < kFxCover)) || info.y == 0) {
+    if (((E != 0 || bad) && (E < 128 || E > 1080 || min(M[0], min(M[1], M[2])) < kFxCover)) || info.y == 0) {
         double tr[12], ti[12];
         hop_fx_fallback<DAG>(in, nb, lk64, N5, lane0, tr, ti);
 #pragma unroll
