@@ -1099,11 +1099,37 @@ k_hop(const HopArgs a) {
 }
 
 // The fixed-point FP64 hop on a domain too small to fill the chip: there a
-// lane's chain of eight directions, ~20 us, is the whole time.  Warp k of a CTA takes direction k of 32 lanes of its tile,
-// and warps 0..5 add the eight directions' half spinors from shared memory,
-// two spin-colour rows each, in the largest of the eight units.
-// 4^4 x 8 (1024 lanes): 20.5 us -> 7.9 with the call's launch.
+// lane's chain of eight directions, ~20 us, is the whole time.  Warp k of a CTA
+// takes direction k of 32 lanes of its tile, and warps 0..5 add the eight
+// directions' half spinors from shared memory, two spin-colour rows each, in
+// the largest of the eight units.  4^4 x 8 (1024 lanes): 20.5 us -> 7.9 with
+// the call's launch.  Lanes that need the FP64 form take it the same way, a
+// direction a warp, its sums in hop_fx_fallback's order.
 constexpr int kSplitLanes = 32;
+
+// transported half spinor of direction k in FP64, into g[(q * 3 + colour) * 2 + part][lane]
+template <bool DAG>
+__device__ __noinline__ void hop_fx_dir64(int k, const double* in, const int* nb, const double* lk, int N5, int lane0,
+                                          long long* g) {
+    double ar[12][1], ai[12][1];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) ar[c][0] = ai[c][0] = 0.0;
+    switch (k) {
+        case 0: hop_dir<0, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai); break;
+        case 1: hop_dir<1, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai); break;
+        case 2: hop_dir<2, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai); break;
+        case 3: hop_dir<3, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai); break;
+        case 4: hop_dir<4, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai); break;
+        case 5: hop_dir<5, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai); break;
+        case 6: hop_dir<6, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai); break;
+        default: hop_dir<7, DAG, double, double, double, 1>(in, nb, lk, N5, lane0, ar, ai);
+    }
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        g[(2 * c) * kSplitLanes] = __double_as_longlong(ar[c][0]);
+        g[(2 * c + 1) * kSplitLanes] = __double_as_longlong(ai[c][0]);
+    }
+}
 
 template <bool DAG, int EPI>
 __global__ void __launch_bounds__(256, 2) k_hop_fx_split(const HopArgs a) {
@@ -1111,6 +1137,7 @@ __global__ void __launch_bounds__(256, 2) k_hop_fx_split(const HopArgs a) {
     __shared__ int s_E[8][kSplitLanes];             // unit, 0: nothing, -1: the FP64 form decides
     __shared__ double s_red[256];
     __shared__ double s_sum[kMaxLanes / 2];
+    __shared__ unsigned s_fp64;                     // lanes that the FP64 form decides
     const int N5 = a.N5, Ls = a.Ls, nrhs = a.nrhs;
     const int4 tl = a.tiles[blockIdx.x];
     const int items = tl.z * N5;
@@ -1160,8 +1187,11 @@ __global__ void __launch_bounds__(256, 2) k_hop_fx_split(const HopArgs a) {
             }
         }
         s_E[k][j] = E;
+        if (threadIdx.x == 0) s_fp64 = 0;
         __syncthreads();
-        double nrm = 0.0;
+        double nrm = 0.0, re[2] = {0.0, 0.0}, im[2] = {0.0, 0.0}, factor = 1.0;
+        const bool upper = k < 3;   // rows 2 k, 2 k + 1: upper spins for k < 3
+        bool fp64 = false;
         if (k < 6 && on) {
             int Em = 0;
             bool bad = false;
@@ -1170,10 +1200,8 @@ __global__ void __launch_bounds__(256, 2) k_hop_fx_split(const HopArgs a) {
                 Em = max(Em, s_E[d][j]);
                 bad |= s_E[d][j] < 0;
             }
-            double re[2], im[2], factor;
-            bool fp64 = ((Em != 0 || bad) && (Em < 128 || Em > 1080)) || info.y == 0;
+            fp64 = ((Em != 0 || bad) && (Em < 128 || Em > 1080)) || info.y == 0;
             if (!fp64) {
-                const bool upper = k < 3;   // rows 2 k, 2 k + 1: upper spins for k < 3
                 long long sr[2] = {0, 0}, si[2] = {0, 0};
                 int size[2] = {0, 0};       // each row's own sum of |g| decides here
 #pragma unroll
@@ -1203,14 +1231,34 @@ __global__ void __launch_bounds__(256, 2) k_hop_fx_split(const HopArgs a) {
                 factor = __hiloint2double(max(Em + info.x - 54, 1) << 20, 0);
                 fp64 = Em != 0 && min(size[0], size[1]) < kFxCover;
             }
-            if (fp64) {
-                double tr[12], ti[12];
-                hop_fx_fallback<DAG>(in, a.nbr + site * 8, a.links64 + site * 144, N5, lane0, tr, ti);
-#pragma unroll
-                for (int c = 0; c < 12; ++c)
-                    if (c >> 1 == k) { re[c & 1] = tr[c]; im[c & 1] = ti[c]; }
+            if (fp64) atomicOr(&s_fp64, 1u << j);
+        }
+        if (__syncthreads_or(fp64)) {   // (the sums above are done with s_g)
+            const bool redo = (s_fp64 >> j) & 1;
+            if (redo)
+                hop_fx_dir64<DAG>(k, in, a.nbr + site * 8, a.links64 + site * 144, N5, lane0, &s_g[k][0][j]);
+            __syncthreads();
+            if (redo && k < 6) {
                 factor = 1.0;
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int c = 2 * k + e, spin = c / 3, col = c - 3 * spin;
+                    re[e] = im[e] = 0.0;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int d = (i >> 1) + 4 * (i & 1), mu = d & 3;
+                        const int q = upper ? spin : (mu < 2 ? 3 - spin : spin - 2);
+                        const double gr = __longlong_as_double(s_g[d][(q * 3 + col) * 2][j]);
+                        const double gi = __longlong_as_double(s_g[d][(q * 3 + col) * 2 + 1][j]);
+                        const bool minus = fx_plus(mu, q) == ((d < 4) == DAG);   // sign of the term (of its im part for i types)
+                        if (upper) { re[e] += gr; im[e] += gi; }
+                        else if (fx_itype(mu)) { re[e] += minus ? gi : -gi; im[e] += minus ? -gr : gr; }
+                        else { re[e] += minus ? -gr : gr; im[e] += minus ? -gi : gi; }
+                    }
+                }
             }
+        }
+        if (k < 6 && on) {
             const double sc = a.scale * factor;
             const int s = lane0 % Ls;
 #pragma unroll
