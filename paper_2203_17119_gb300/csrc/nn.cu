@@ -603,10 +603,12 @@ __global__ void k_mix_weights(const float* __restrict__ w1, const float* __restr
     }
 }
 
-// Rebuild the mixing matrices after the master weights changed, on stream s;
-// every caller waits for s before it returns, so that a later call may use
-// them on any stream.
+// Rebuild the mixing matrices after the master weights changed, on stream s:
+// first wait for the device, since applications queued on other streams still
+// read them.  Every caller waits for s before it returns, so that a later call
+// may use them on any stream.
 static dwf_status refresh_mix(dwf_nn* K, cudaStream_t s) {
+    DWF_CUDA(cudaDeviceSynchronize());
     MixDirs md{};
     MixOut mo{};
     for (int p = 0; p < 2; ++p) {
