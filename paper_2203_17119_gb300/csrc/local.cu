@@ -88,7 +88,25 @@ __device__ __forceinline__ void shift_sum(float c0, float c1, const float (&x)[V
     }
 }
 
-template <class Sin, class Sin2, class Sout, int VL, int KIND>
+// The thread's lanes of a row: vectors of 16 bytes (8 for two BF16 lanes), or
+// one complex number at a time (WIDE false) for fields aligned only to that.
+template <class S, int VL, bool WIDE>
+__device__ __forceinline__ void load_row(const S* p, float (&re)[VL], float (&im)[VL]) {
+    if constexpr (WIDE) load_lanes<S, VL, float>(p, re, im);
+    else
+#pragma unroll
+        for (int v = 0; v < VL; ++v) load_lanes<S, 1, float>(p + 2 * v, re + v, im + v);
+}
+
+template <class S, int VL, bool WIDE>
+__device__ __forceinline__ void store_row(S* p, const float (&re)[VL], const float (&im)[VL]) {
+    if constexpr (WIDE) store_lanes<S, VL, float>(p, re, im);
+    else
+#pragma unroll
+        for (int v = 0; v < VL; ++v) store_lanes<S, 1, float>(p + 2 * v, re + v, im + v);
+}
+
+template <class Sin, class Sin2, class Sout, int VL, int KIND, bool WIDE>
 __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
     constexpr bool INV = KIND == K_INV || KIND == K_INVR, REV = KIND == K_INVR;
     constexpr int kU = KIND == K_ONE || INV ? 4 : 2;
@@ -149,9 +167,9 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
 #pragma unroll
             for (int v = 0; v < VL; ++v) xr[u][v] = xi[u][v] = zr[u][v] = zi[u][v] = 0.f;
             if (ok) {
-                if (KIND == K_PB) load_lanes<float, VL, float>(a.cg_p + 2 * g, xr[u], xi[u]);
-                else load_lanes<Sin, VL, float>(in + 2 * g, xr[u], xi[u]);
-                if (KIND == K_PB || KIND == K_POST) load_lanes<Sin2, VL, float>(in2 + 2 * g, zr[u], zi[u]);
+                if (KIND == K_PB) load_row<float, VL, WIDE>(a.cg_p + 2 * g, xr[u], xi[u]);
+                else load_row<Sin, VL, WIDE>(in + 2 * g, xr[u], xi[u]);
+                if (KIND == K_PB || KIND == K_POST) load_row<Sin2, VL, WIDE>(in2 + 2 * g, zr[u], zi[u]);
             }
         }
         float pn = 0.f;
@@ -172,7 +190,7 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
                         xi[u][v] = fmaf(coef, xi[u][v], zi[u][v]);
                     }
                 }
-                if (ok && live) store_lanes<float, VL, float>(a.cg_p + 2 * g, xr[u], xi[u]);
+                if (ok && live) store_row<float, VL, WIDE>(a.cg_p + 2 * g, xr[u], xi[u]);
             }
             if (INV) {
                 // mirrored lanes for S_+ (K_INVR: for S_-): m runs with the recurrence
@@ -244,11 +262,11 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
             if (!ok) continue;
             if (cg) {   // x += alpha p, r -= alpha y
                 float rr[VL], ri[VL];
-                load_lanes<float, VL, float>(a.cg_r + 2 * g, rr, ri);
+                load_row<float, VL, WIDE>(a.cg_r + 2 * g, rr, ri);
                 if (live) {
                     float pr[VL], pi[VL], vr[VL], vi[VL];
-                    load_lanes<float, VL, float>(a.cg_p + 2 * g, pr, pi);
-                    load_lanes<float, VL, float>(a.cg_x + 2 * g, vr, vi);
+                    load_row<float, VL, WIDE>(a.cg_p + 2 * g, pr, pi);
+                    load_row<float, VL, WIDE>(a.cg_x + 2 * g, vr, vi);
 #pragma unroll
                     for (int v = 0; v < VL; ++v) {
                         vr[v] = fmaf(coef, pr[v], vr[v]);
@@ -256,8 +274,8 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
                         rr[v] = fmaf(-coef, yr[v], rr[v]);
                         ri[v] = fmaf(-coef, yi[v], ri[v]);
                     }
-                    store_lanes<float, VL, float>(a.cg_x + 2 * g, vr, vi);
-                    store_lanes<float, VL, float>(a.cg_r + 2 * g, rr, ri);
+                    store_row<float, VL, WIDE>(a.cg_x + 2 * g, vr, vi);
+                    store_row<float, VL, WIDE>(a.cg_r + 2 * g, rr, ri);
                 }
 #pragma unroll
                 for (int v = 0; v < VL; ++v) { yr[v] = rr[v]; yi[v] = ri[v]; }
@@ -266,16 +284,16 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
                     float ur[VL], ui[VL], vr[VL], vi[VL];
 #pragma unroll
                     for (int v = 0; v < VL; ++v) vr[v] = vi[v] = 0.f;
-                    load_lanes<Sout, VL, float>(reinterpret_cast<const Sout*>(a.lin_u) + 2 * g, ur, ui);
+                    load_row<Sout, VL, WIDE>(reinterpret_cast<const Sout*>(a.lin_u) + 2 * g, ur, ui);
                     if (a.lin_v != nullptr)
-                        load_lanes<Sout, VL, float>(reinterpret_cast<const Sout*>(a.lin_v) + 2 * g, vr, vi);
+                        load_row<Sout, VL, WIDE>(reinterpret_cast<const Sout*>(a.lin_v) + 2 * g, vr, vi);
 #pragma unroll
                     for (int v = 0; v < VL; ++v) {
                         yr[v] = fmaf(a.lin_a, yr[v], fmaf(a.lin_bu, ur[v], a.lin_bv * vr[v]));
                         yi[v] = fmaf(a.lin_a, yi[v], fmaf(a.lin_bu, ui[v], a.lin_bv * vi[v]));
                     }
                 }
-                store_lanes<Sout, VL, float>(reinterpret_cast<Sout*>(a.out) + 2 * g, yr, yi);
+                store_row<Sout, VL, WIDE>(reinterpret_cast<Sout*>(a.out) + 2 * g, yr, yi);
             }
 #pragma unroll
             for (int v = 0; v < VL; ++v) pn = fmaf(yr[v], yr[v], fmaf(yi[v], yi[v], pn));
@@ -289,7 +307,7 @@ __global__ void __launch_bounds__(kLocalThreads) k_local(const LocalArgs a) {
     }
 }
 
-template <class Sin, class Sin2, class Sout, int VL>
+template <class Sin, class Sin2, class Sout, int VL, bool WIDE>
 static dwf_status launch_vl(dwf_handle* h, const LocalCall& c, const TileSet& ts, cudaStream_t s) {
     const FiveD& f = h->f5[0];
     const int nt = ts.ntiles[c.parity];
@@ -316,7 +334,7 @@ static dwf_status launch_vl(dwf_handle* h, const LocalCall& c, const TileSet& ts
     a.alpha = c.alpha;
     a.run = c.run;
     a.partial = c.partial;
-    void (*kern)(const LocalArgs) = k_local<Sin, Sin2, Sout, VL, K_ONE>;
+    void (*kern)(const LocalArgs) = k_local<Sin, Sin2, Sout, VL, K_ONE, WIDE>;
     switch (c.op) {
         case L_MINV:
         case L_BMINV: {
@@ -330,7 +348,7 @@ static dwf_status launch_vl(dwf_handle* h, const LocalCall& c, const TileSet& ts
             else a.wall = (float)(f.mf / (1.0 + f.mf * rL));
             a.c0 = (float)(c.scale * f.inv_d * (c.op == L_BMINV ? f.b5 : 1.0));
             a.c1 = (float)(c.op == L_BMINV ? c.scale * f.inv_d * f.c5 : 0.0);
-            kern = rev ? k_local<Sin, Sin2, Sout, VL, K_INVR> : k_local<Sin, Sin2, Sout, VL, K_INV>;
+            kern = rev ? k_local<Sin, Sin2, Sout, VL, K_INVR, WIDE> : k_local<Sin, Sin2, Sout, VL, K_INV, WIDE>;
             break;
         }
         case L_POST:
@@ -345,12 +363,12 @@ static dwf_status launch_vl(dwf_handle* h, const LocalCall& c, const TileSet& ts
                 a.lin_bu = (float)c.lin->bu;
                 a.lin_bv = (float)c.lin->bv;
             }
-            kern = k_local<Sin, Sin2, Sout, VL, K_POST>;
+            kern = k_local<Sin, Sin2, Sout, VL, K_POST, WIDE>;
             break;
         case L_PB:
             a.c0 = (float)f.b5;
             a.c1 = (float)f.c5;
-            kern = k_local<Sin, Sin2, Sout, VL, K_PB>;
+            kern = k_local<Sin, Sin2, Sout, VL, K_PB, WIDE>;
             break;
         default:
             a.c0 = (float)(c.op == L_MOOEE ? f.d : c.op == L_B ? f.b5 : 1.0);
@@ -362,11 +380,17 @@ static dwf_status launch_vl(dwf_handle* h, const LocalCall& c, const TileSet& ts
     return DWF_OK;
 }
 
-// 4 lanes per thread where Ls allows it (fewer shuffles a lane), else 2.
+// 4 lanes per thread where Ls allows it (fewer shuffles a lane), else 2; fields
+// off the 16-byte boundaries that the vectors need (an operator's caller may
+// pass a view) go number by number.
 template <class Sin, class Sin2, class Sout>
 static dwf_status launch_t(dwf_handle* h, const LocalCall& c, const TileSet& ts, cudaStream_t s) {
-    if (h->p.Ls % 4 == 0) return launch_vl<Sin, Sin2, Sout, 4>(h, c, ts, s);
-    return launch_vl<Sin, Sin2, Sout, 2>(h, c, ts, s);
+    const void* all[] = {c.in, c.in2, c.out, c.cg_x, c.cg_r, c.cg_p, c.lin ? c.lin->u : nullptr, c.lin ? c.lin->v : nullptr};
+    uintptr_t off = 0;
+    for (const void* q : all) off |= reinterpret_cast<uintptr_t>(q);
+    if (off % 16 != 0) return launch_vl<Sin, Sin2, Sout, 2, false>(h, c, ts, s);
+    if (h->p.Ls % 4 == 0) return launch_vl<Sin, Sin2, Sout, 4, true>(h, c, ts, s);
+    return launch_vl<Sin, Sin2, Sout, 2, true>(h, c, ts, s);
 }
 
 // The right-hand side counts the site-local operators take: the solver's
