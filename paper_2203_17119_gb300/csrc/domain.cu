@@ -207,85 +207,95 @@ dwf_status set_tile_order(dwf_handle* h, int order, int bz, int bt) {
 // ----------------------------------------------------------- link tables
 // doubled link table of one parity: [site][k][3][3] complex, k < 4 forward
 // U_mu(x), k >= 4 backward U_mu(x - mu)^+; zero where src < 0 (cut).
-__global__ void k_gather_links(const double* __restrict__ U, const int64_t* __restrict__ src,
-                               int64_t n /* sites * 8 */, double* __restrict__ l64,
-                               float* __restrict__ l32, bf16* __restrict__ l16) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n * 9;
-         i += (int64_t)gridDim.x * blockDim.x) {
+//
+// The FP64 hop's fixed-point form: w = (hi 2^32 + lo) 2^(exp - 61), lo a signed
+// word above -2^31, with |w| < 1.125 2^exp for every link.  Links are SU(3) in
+// earnest, so one pass writes the tables with exp = kFxExp and finds the
+// largest element; set_gauge repeats it with another exp where that one does
+// not fit.
+//
+// Bound by memory: a link is read twice and written in 16 + 8 + 4 + 16 bytes a
+// complex number.  dwf_set_gauge on 4^4 / 16^4 / 32^4 sites: 27 / 68 / 623 us
+// without the fixed-point table, 53 / 162 / 1449 with it formed from the FP64
+// table in four passes of its own, 28 / 87 / 902 this way.
+struct LinkArgs {
+    const double* U;
+    const int64_t* src[2];    // [site][k] link, or -1
+    int64_t n[2];             // sites * 8
+    double2* l64[2];
+    float2* l32[2];
+    __nv_bfloat162* l16[2];
+    int4* fx[2];              // (re high, re low, im high, im low)
+    int exp;
+    int* top;                 // high word of the largest |element|
+};
+
+constexpr int kFxExp = 0;
+
+// w 2^(61 - exp) to the nearest integer (ties to even), |w| < 4 2^exp; in integer
+// arithmetic, since two more FP64 operations a number would bound the pass
+// (with them 32^4 took 1060 us)
+__device__ __forceinline__ int2 fx_link(double w, int exp) {
+    const int h = __double2hiint(w), e = (h >> 20) & 0x7ff;
+    const unsigned long long m = ((unsigned long long)((h & 0xfffff) | (e > 0 ? 0x100000 : 0)) << 32) | (uint32_t)__double2loint(w);
+    const int sh = max(e, 1) - 1014 - exp;   // w = m 2^(max(e, 1) - 1075)
+    unsigned long long u;
+    if (sh >= 0) u = m << min(sh, 10);
+    else {
+        const int r = min(-sh, 60);
+        u = (m + ((1ull << (r - 1)) - 1) + ((m >> r) & 1)) >> r;
+    }
+    const long long v = h < 0 ? -(long long)u : (long long)u;
+    // the low word is negated for conjugates: -2^31 becomes its neighbour (2^-61 off)
+    return make_int2((int)((v + (1ll << 31)) >> 32), max((int)v, -2147483647));
+}
+
+__global__ void __launch_bounds__(256) k_gather_links(const LinkArgs a) {
+    __shared__ int s_top;
+    if (threadIdx.x == 0) s_top = 0;
+    __syncthreads();
+    int top = 0;
+    const int64_t n0 = a.n[0] * 9, nall = n0 + a.n[1] * 9;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nall; t += (int64_t)gridDim.x * blockDim.x) {
+        const int p = t >= n0;
+        const int64_t i = p ? t - n0 : t;
         const int64_t sk = i / 9;
-        const int ab = (int)(i % 9);
-        const int a = ab / 3, b = ab % 3;
-        const int k = (int)(sk % 8);
-        const int64_t g = src[sk];
+        const int ab = (int)(i - sk * 9);
+        const int64_t g = a.src[p][sk];
         double re = 0.0, im = 0.0;
         if (g >= 0) {
-            if (k < 4) {
-                re = U[(g * 9 + a * 3 + b) * 2];
-                im = U[(g * 9 + a * 3 + b) * 2 + 1];
-            } else {   // (U^+)_{ab} = conj(U_{ba})
-                re = U[(g * 9 + b * 3 + a) * 2];
-                im = -U[(g * 9 + b * 3 + a) * 2 + 1];
-            }
+            const bool fwd = (sk & 7) < 4;
+            const int e = fwd ? ab : ab % 3 * 3 + ab / 3;   // backward: (U^+)_{ab} = conj(U_{ba})
+            re = a.U[(g * 9 + e) * 2];
+            im = a.U[(g * 9 + e) * 2 + 1];
+            if (!fwd) im = -im;
         }
-        l64[2 * i] = re;
-        l64[2 * i + 1] = im;
-        l32[2 * i] = (float)re;
-        l32[2 * i + 1] = (float)im;
-        l16[2 * i] = __float2bfloat16_rn((float)re);
-        l16[2 * i + 1] = __float2bfloat16_rn((float)im);
+        a.l64[p][i] = make_double2(re, im);
+        a.l32[p][i] = make_float2((float)re, (float)im);
+        a.l16[p][i] = __floats2bfloat162_rn((float)re, (float)im);
+        const int2 r = fx_link(re, a.exp), m = fx_link(im, a.exp);
+        a.fx[p][i] = make_int4(r.x, r.y, m.x, m.y);
+        top = max(top, max(__double2hiint(re) & 0x7fffffff, __double2hiint(im) & 0x7fffffff));
     }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_top > *(volatile int*)a.top) atomicMax(a.top, s_top);
 }
 
-// Range of the links' sizes: the biased exponents of the largest element of
-// any link, and of the smallest link's largest element (links of zeros aside);
-// an element up to 1.125 2^k counts as below 2^k (unit links, and 1 + rounding,
-// then take the unit of the links within them); a NaN or infinity has exponent 2046 or 2047.
-__global__ void k_link_range(const double* __restrict__ l64, int64_t n /* sites * 8 */, int* __restrict__ range) {
-    int hi = 0, lo = 4096;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int e = 0;
-#pragma unroll
-        for (int j = 0; j < 18; ++j) e = max(e, ((__double2hiint(l64[i * 18 + j]) & 0x7fffffff) - 0x20000) >> 20);
-        if (e > 0) {
-            hi = max(hi, e);
-            lo = min(lo, e);
-        }
-    }
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(&range[0], hi);
-        atomicMin(&range[1], lo);
-    }
-}
-
-// Fixed-point links: w = (hi 2^32 + lo) 2^(exp - 61), lo a signed word above
-// -2^31, with |w| < 1.125 2^exp.  Covered (info[1] = 1): finite links whose sizes differ by at
-// most 2^8, so that the common unit costs none of them precision against FP64
-// (SU(3) links lie within a factor sqrt(3)), of a size that leaves the
-// result's exponent in range.
-__device__ __forceinline__ bool fx_covered(const int* range, int* exp) {
-    *exp = range[0] - 1022;
-    return range[0] > 0 && range[0] - range[1] <= 8 && *exp >= -32 && *exp <= 32;
-}
-
-__global__ void k_fix_links(const double* __restrict__ l64, int64_t n /* reals */, const int* __restrict__ range,
-                            int2* __restrict__ fx) {
-    int exp;
-    if (!fx_covered(range, &exp)) return;
-    const double scale = __hiloint2double((1023 + 61 - exp) << 20, 0);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const long long v = __double2ll_rn(l64[i] * scale);
-        // the low word is negated for conjugates: -2^31 becomes its neighbour (2^-61 off)
-        fx[i] = make_int2((int)((v + (1ll << 31)) >> 32), max((int)v, -2147483647));
-    }
-}
-
-__global__ void k_fx_info(const int* __restrict__ range, int* __restrict__ info) {
-    int exp;
-    const bool ok = fx_covered(range, &exp);
-    info[0] = ok ? exp : 0;
-    info[1] = ok ? 1 : 0;
+// info = {exp, 1 if the table with it covers links up to `top`, the exp that
+// fits them, 1 if there is one}, also to the host.  An element up to 1.125 2^k counts as below
+// 2^k: unit links, and 1 + rounding, keep exp = 0.  A table may be one bit
+// coarser than the links need; links beyond 2^+-32, or not finite, have none.
+// Uneven links need no rule: a lane that only small ones reach runs the FP64 form.
+__global__ void k_fx_info(const int* __restrict__ top, int exp, int* __restrict__ info, int* __restrict__ host) {
+    const int fit = ((*top - 0x20000) >> 20) - 1022;
+    const bool ok = *top > 0 && fit >= -32 && fit <= 32;
+    const bool here = ok && fit <= exp && exp <= fit + 1;
+    info[0] = host[0] = exp;
+    info[1] = host[1] = here ? 1 : 0;
+    host[2] = fit;
+    host[3] = ok ? 1 : 0;
 }
 
 // --------------------------------------------------------- layout kernels
@@ -370,38 +380,34 @@ dwf_status unpack(dwf_handle* h, double* dst, const void* src, int nrhs, dwf_pre
 }
 
 dwf_status set_gauge(dwf_handle* h, const double* U, cudaStream_t s) {
+    LinkArgs a{};
+    a.U = U;
     for (int p = 0; p < 2; ++p) {
-        const int64_t n = h->nsite[p] * 8;
-        if (n == 0) continue;
-        const int64_t blocks = std::min<int64_t>((n * 9 + 255) / 256, 152 * 64);
-        k_gather_links<<<(int)blocks, 256, 0, s>>>(U, h->d_link_src[p], n, (double*)h->d_links[0][p],
-                                                   (float*)h->d_links[1][p], (bf16*)h->d_links[2][p]);
-        note_launch();
-        DWF_CUDA(cudaGetLastError());
+        a.src[p] = h->d_link_src[p];
+        a.n[p] = h->nsite[p] * 8;
+        a.l64[p] = (double2*)h->d_links[0][p];
+        a.l32[p] = (float2*)h->d_links[1][p];
+        a.l16[p] = (__nv_bfloat162*)h->d_links[2][p];
+        a.fx[p] = (int4*)h->d_links_fx[p];
     }
-    // the fixed-point table, where the links' sizes allow it
-    int* range = h->d_fx_info + 2;
-    const int none[2] = {0, 4096};
-    DWF_CUDA(cudaMemcpyAsync(range, none, sizeof(none), cudaMemcpyHostToDevice, s));
-    for (int pass = 0; pass < 2; ++pass)
-        for (int p = 0; p < 2; ++p) {
-            const int64_t n = h->nsite[p] * 8;
-            if (n == 0) continue;
-            const double* l64 = (const double*)h->d_links[0][p];
-            if (pass == 0)
-                k_link_range<<<(int)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(l64, n, range);
-            else
-                k_fix_links<<<(int)std::min<int64_t>((n * 18 + 255) / 256, 152 * 32), 256, 0, s>>>(
-                    l64, n * 18, range, (int2*)h->d_links_fx[p]);
+    a.exp = kFxExp;
+    a.top = h->d_fx_info + 2;
+    const int64_t n = a.n[0] + a.n[1];
+    const int* info = h->fx_info_host;
+    for (int pass = 0; pass < 2; ++pass) {
+        DWF_CUDA(cudaMemsetAsync(a.top, 0, sizeof(int), s));
+        if (n > 0) {
+            k_gather_links<<<(int)std::min<int64_t>((n * 9 + 255) / 256, 152 * 64), 256, 0, s>>>(a);
             note_launch();
             DWF_CUDA(cudaGetLastError());
         }
-    k_fx_info<<<1, 1, 0, s>>>(range, h->d_fx_info);
-    note_launch();
-    DWF_CUDA(cudaGetLastError());
-    int info[2] = {0, 0};
-    DWF_CUDA(cudaMemcpyAsync(info, h->d_fx_info, sizeof(info), cudaMemcpyDeviceToHost, s));
-    DWF_CUDA(cudaStreamSynchronize(s));
+        k_fx_info<<<1, 1, 0, s>>>(a.top, a.exp, h->d_fx_info, h->fx_info_host);
+        note_launch();
+        DWF_CUDA(cudaGetLastError());
+        DWF_CUDA(cudaStreamSynchronize(s));
+        if (info[1] != 0 || info[3] == 0) break;
+        a.exp = info[2];
+    }
     h->fx_links = info[1] != 0;
     h->have_gauge = true;
     return DWF_OK;
@@ -600,6 +606,10 @@ dwf_status create(dwf_handle** out, const dwf_params* p, const dwf_box* boxes, i
     if (st == DWF_OK) st = init_hop_kernels();
     if (st == DWF_OK) st = init_hop_tc_kernels();
     if (st == DWF_OK) st = dalloc(&h->d_fx_info, 4);
+    if (st == DWF_OK && cudaMallocHost(&h->fx_info_host, 4 * sizeof(int)) != cudaSuccess) {
+        set_error("dwf_create: page-locked memory failed");
+        st = DWF_ERR_CUDA;
+    }
     if (st == DWF_OK) st = dalloc(&h->d_err, 1);
     if (st == DWF_OK) {
         if (cudaMemset(h->d_err, 0, sizeof(int)) != cudaSuccess) {
@@ -723,6 +733,7 @@ dwf_status destroy(dwf_handle* h) {
         cudaFree(h->d_links_fx[q]);
     }
     cudaFree(h->d_fx_info);
+    cudaFreeHost(h->fx_info_host);
     cudaFree(h->d_box_canon_vol);
     cudaFree(h->d_err);
     cudaFree(h->d_tmp);

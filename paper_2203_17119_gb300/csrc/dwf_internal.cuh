@@ -160,9 +160,11 @@ struct dwf_handle {
     void* d_links[3][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};
     // fixed-point form of the FP64 table (hop.cu): [site][8][9] x (re, im) x
     // (high, low) int32, in units 2^(exponent - 61).  d_fx_info: exponent, 1 if
-    // the loaded links are covered by it, and their size range (set_gauge).
+    // the loaded links are covered by it, and the largest element (set_gauge);
+    // fx_info_host: what of it the host decides by, page-locked.
     int* d_links_fx[2] = {nullptr, nullptr};
     int* d_fx_info = nullptr;
+    int* fx_info_host = nullptr;
     bool fx_links = false;
     bool have_gauge = false;
     std::map<int, dwf::TileSet> tiles;

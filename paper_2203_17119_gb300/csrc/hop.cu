@@ -400,8 +400,8 @@ __device__ __forceinline__ void hop_dir(const Sin* __restrict__ in, const int* s
 // the FP64 form -- numbers that a larger one does not reach: links that do not
 // mix two colours, a neighbour that the projector annihilates, one neighbour
 // far above the others --, and so do a NaN, an infinity, all components below
-// 2^-895 or one above 2^56, and a handle whose links differ in size by more
-// than 2^8 (set_gauge).  A warp with one such lane takes some 25 us longer, a
+// 2^-895 or one above 2^56, and a handle whose links are not finite or beyond
+// 2^+-32 (set_gauge).  A warp with one such lane takes some 25 us longer, a
 // fixed tail on small lattices: with the smallest |g| of all six components in
 // one sum, one Gaussian lane in 10^5 failed, and 16^4 x 12 took 233 to 245 us
 // instead of 217.  Telling them costs 3% of the bare hop (16^4 x 12 209 -> 217
