@@ -133,7 +133,9 @@ typedef struct dwf_mg dwf_mg;
  * Dirichlet blocks D_Omega of `nbox` boxes (Sec. 2.1, Sec. 2.4).  Builds the
  * site lists, neighbour tables and tile tables on the host and allocates all
  * device workspace for up to `nrhs_max` right-hand sides, on the current
- * CUDA device.  Errors: DWF_ERR_ARG (Lx odd, Ls < 1, extents out of range,
+ * CUDA device; last the fixed-point links of the FP64 hop, 1152 bytes a site,
+ * without which, where they no longer fit, that hop runs about three times
+ * slower.  Errors: DWF_ERR_ARG (Lx odd, Ls < 1, extents out of range,
  * nrhs_max < 1 or Ls * nrhs_max > 256), DWF_ERR_CUDA (allocation). */
 dwf_status dwf_create(dwf_handle** h, const dwf_params* p, const dwf_box* boxes,
                       int nbox, int nrhs_max);

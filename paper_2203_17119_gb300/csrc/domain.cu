@@ -273,8 +273,10 @@ __global__ void __launch_bounds__(256) k_gather_links(const LinkArgs a) {
         a.l64[p][i] = make_double2(re, im);
         a.l32[p][i] = make_float2((float)re, (float)im);
         a.l16[p][i] = __floats2bfloat162_rn((float)re, (float)im);
-        const int2 r = fx_link(re, a.exp), m = fx_link(im, a.exp);
-        a.fx[p][i] = make_int4(r.x, r.y, m.x, m.y);
+        if (a.fx[p] != nullptr) {
+            const int2 r = fx_link(re, a.exp), m = fx_link(im, a.exp);
+            a.fx[p][i] = make_int4(r.x, r.y, m.x, m.y);
+        }
         top = max(top, max(__double2hiint(re) & 0x7fffffff, __double2hiint(im) & 0x7fffffff));
     }
     top = __reduce_max_sync(0xffffffffu, top);
@@ -394,6 +396,7 @@ dwf_status set_gauge(dwf_handle* h, const double* U, cudaStream_t s) {
     a.top = h->d_fx_info + 2;
     const int64_t n = a.n[0] + a.n[1];
     const int* info = h->fx_info_host;
+    const bool table = h->d_links_fx[0] != nullptr;
     for (int pass = 0; pass < 2; ++pass) {
         DWF_CUDA(cudaMemsetAsync(a.top, 0, sizeof(int), s));
         if (n > 0) {
@@ -405,10 +408,10 @@ dwf_status set_gauge(dwf_handle* h, const double* U, cudaStream_t s) {
         note_launch();
         DWF_CUDA(cudaGetLastError());
         DWF_CUDA(cudaStreamSynchronize(s));
-        if (info[1] != 0 || info[3] == 0) break;
+        if (info[1] != 0 || info[3] == 0 || !table) break;
         a.exp = info[2];
     }
-    h->fx_links = info[1] != 0;
+    h->fx_links = table && info[1] != 0;
     h->have_gauge = true;
     return DWF_OK;
 }
@@ -594,7 +597,6 @@ dwf_status create(dwf_handle** out, const dwf_params* p, const dwf_box* boxes, i
         if (st == DWF_OK) h->site_local_host[q] = site_local[q];
         for (int pr = 0; pr < 3 && st == DWF_OK; ++pr)
             st = dalloc((char**)&h->d_links[pr][q], ns * 144 * prec_size((dwf_prec)pr));
-        if (st == DWF_OK) st = dalloc(&h->d_links_fx[q], ns * 288);
     }
     if (st == DWF_OK) {
         std::vector<int64_t> bv(2 * h->nbox);
@@ -631,6 +633,15 @@ dwf_status create(dwf_handle** out, const dwf_params* p, const dwf_box* boxes, i
         st = get_tiles(h, h->default_T, &ts);
     }
     if (st == DWF_OK) {
+        // the fixed-point links last: where they do not fit any more, the FP64 hop
+        // runs its FP64 form
+        for (int q = 0; q < 2; ++q)
+            if (dev_malloc(&h->d_links_fx[q], std::max<size_t>(h->nsite[q], 1) * 288 * sizeof(int)) != cudaSuccess) {
+                cudaGetLastError();
+                cudaFree(h->d_links_fx[0]);
+                h->d_links_fx[0] = h->d_links_fx[1] = nullptr;
+                break;
+            }
         cudaError_t e = cudaDeviceSynchronize();
         if (e != cudaSuccess) {
             set_error("dwf_create: %s", cudaGetErrorString(e));
