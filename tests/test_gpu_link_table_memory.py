@@ -20,7 +20,7 @@ def test_created_without_the_table():
         return G.Handle(dims, Ls, G.Action(1.8, 0.01))
 
     g = torch.Generator(device="cuda").manual_seed(8)
-    U = torch.linalg.qr(torch.randn(sites * 4, 3, 3, dtype=torch.complex128, device="cuda", generator=g))[0].reshape(-1)
+    U = 0.2 * torch.randn(sites * 4 * 9, dtype=torch.complex128, device="cuda", generator=g)   # (any links serve)
     h = handle()
     h.set_gauge(U)
     src = h.empty_cb(1)
