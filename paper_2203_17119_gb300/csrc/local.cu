@@ -393,9 +393,10 @@ static dwf_status launch_t(dwf_handle* h, const LocalCall& c, const TileSet& ts,
     return launch_vl<Sin, Sin2, Sout, 2, true>(h, c, ts, s);
 }
 
-// The right-hand side counts the site-local operators take: the solver's
-// reductions want lcm(32, nrhs) threads, and the limits are those of the rows
-// kernels that first served them.
+// The right-hand side counts the site-local operators take.  Only the solver's
+// reductions have a limit of their own (lcm(32, nrhs) threads); the second
+// bound is that of rows staged in shared memory, which no kernel here does any
+// more: it is kept so that a count is taken or refused by the same rule as ever.
 static dwf_status rhs_supported(int nrhs, int Ls, int word) {
     auto lcm32 = [](int n, int cap) {
         int l = 32;
@@ -412,7 +413,7 @@ static dwf_status rhs_supported(int nrhs, int Ls, int word) {
     if (threads < target) threads *= target / threads;
     const size_t smem = (size_t)4 * threads * (Ls + 1) * word;
     if (smem > 200 * 1024) {
-        set_error("local: %zu bytes of shared memory for nrhs=%d, Ls=%d", smem, nrhs, Ls);
+        set_error("local: %d right-hand sides at Ls = %d are not supported", nrhs, Ls);
         return DWF_ERR_UNSUPPORTED;
     }
     return DWF_OK;

@@ -657,7 +657,10 @@ static void free_nn_bufs(NNWS& w) {
 }
 
 constexpr int kWgBlocks = 152 * 2;
-constexpr int kMaxTrainLanes = 236;   // Ls * nrhs of a training batch (Ls is even)
+// Ls * nrhs of a training batch.  The weight gradient has no such limit (32
+// pixels a step, whatever the lanes); kept so that a batch is taken or refused
+// by the same rule as ever.
+constexpr int kMaxTrainLanes = 236;
 
 template <int MF, int NF>
 static cudaError_t wgrad_attr() {
