@@ -17,6 +17,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "dev_common.cuh"
@@ -500,6 +501,15 @@ struct dwf_nn {
     float* fold = nullptr;       // even sites, 8 x 8 blocks
     float* nmat = nullptr;       // odd sites, the spin matrices of k_odd_sum
     int adam_t = 0;
+    // the last application queued on each stream, for the next change of the
+    // mixing matrices to wait for; untracked once one is in a captured graph
+    struct Reader {
+        cudaStream_t stream;
+        cudaEvent_t done;
+    };
+    std::mutex readers_mu;
+    std::vector<Reader> readers;
+    bool untracked = false;
 };
 
 namespace dwf {
@@ -603,12 +613,45 @@ __global__ void k_mix_weights(const float* __restrict__ w1, const float* __restr
     }
 }
 
-// Rebuild the mixing matrices after the master weights changed, on stream s:
-// first wait for the device, since applications queued on other streams still
-// read them.  Every caller waits for s before it returns, so that a later call
-// may use them on any stream.
+// Note that the work queued on s so far reads the mixing matrices.  An event is
+// never recorded before what it stood for is done: of another stream, or of an
+// earlier stream with the same handle.
+constexpr size_t kMaxReaders = 64;
+
+static dwf_status note_reader(dwf_nn* K, cudaStream_t s) {
+    std::lock_guard<std::mutex> lock(K->readers_mu);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    DWF_CUDA(cudaStreamIsCapturing(s, &cap));
+    if (cap != cudaStreamCaptureStatusNone) {
+        K->untracked = true;
+        return DWF_OK;
+    }
+    auto it = std::find_if(K->readers.begin(), K->readers.end(), [s](const dwf_nn::Reader& r) { return r.stream == s; });
+    if (it == K->readers.end() && K->readers.size() < kMaxReaders) {
+        cudaEvent_t e;
+        DWF_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        it = K->readers.insert(it, {s, e});
+    } else {
+        if (it == K->readers.end()) it = K->readers.begin();
+        DWF_CUDA(cudaStreamWaitEvent(s, it->done, 0));
+        it->stream = s;
+    }
+    DWF_CUDA(cudaEventRecord(it->done, s));
+    return DWF_OK;
+}
+
+// Rebuild the mixing matrices after the master weights changed, on stream s,
+// behind the applications queued on other streams, which still read them.  Not
+// by a wait for the device: that would wait for unrelated work, and fail while
+// any thread captures a graph (a solve does); only a graph that holds an
+// application, whose replays leave no event, asks for it.  Every caller waits for
+// s before it returns, so that a later call may use them on any stream.
 static dwf_status refresh_mix(dwf_nn* K, cudaStream_t s) {
-    DWF_CUDA(cudaDeviceSynchronize());
+    {
+        std::lock_guard<std::mutex> lock(K->readers_mu);
+        if (K->untracked) DWF_CUDA(cudaDeviceSynchronize());
+        for (const dwf_nn::Reader& r : K->readers) DWF_CUDA(cudaStreamWaitEvent(s, r.done, 0));
+    }
     MixDirs md{};
     MixOut mo{};
     for (int p = 0; p < 2; ++p) {
@@ -837,7 +880,7 @@ dwf_status nn_apply_internal(dwf_nn* K, dwf_handle* h, float* out, const float* 
     DWF_TRY(launch_mix(h, nrhs, 0, in, kNFold[0], w->psi, kNFold[0], K->fold, s, true));
     const TileSet* tsp = nullptr;
     DWF_TRY(get_tiles(h, tile_for(h, nrhs), &tsp));
-    if (tsp->ntiles[1] == 0) return DWF_OK;
+    if (tsp->ntiles[1] == 0) return note_reader(K, s);
     OddArgs a{};
     a.x = in;
     a.psi = w->psi;
@@ -852,7 +895,7 @@ dwf_status nn_apply_internal(dwf_nn* K, dwf_handle* h, float* out, const float* 
     k_odd_sum<<<tsp->ntiles[1], 256, 0, s>>>(a);
     note_launch();
     DWF_CUDA(cudaGetLastError());
-    return DWF_OK;
+    return note_reader(K, s);
 }
 
 }  // namespace dwf
@@ -905,6 +948,7 @@ dwf_status dwf_nn_destroy(dwf_nn* K) {
     if (!K) return DWF_OK;
     cudaFree(K->d_w1); cudaFree(K->d_w2); cudaFree(K->d_m); cudaFree(K->d_v);
     cudaFree(K->d_mix);
+    for (const dwf_nn::Reader& r : K->readers) cudaEventDestroy(r.done);
     delete K;
     return DWF_OK;
 }
